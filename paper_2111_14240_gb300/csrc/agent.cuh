@@ -9,7 +9,8 @@
 //   S2  A = F a                 (2-D DFT)
 //   S3  A' = y_j A / |A|, 0 where A = 0   (Section III-A)
 //   S4  w_j = (alpha v_j + D^-1 F^* A') / (1 + alpha)   (equation F-interpolate)
-//   S5  u_j = 2 w_j - v_j (input of G), q_j <- v_j - 2 rho_cur w_j
+//   S5  q_j <- v_j - 2 rho_cur w_j, and u_j = 2 w_j - v_j (input of G) where
+//       the consensus is not taken from q (consensus_from_q)
 // and per-CTA FP64 partial sums of |z - w|^2, |w|^2, (y - |A|)^2, y^2.
 //
 // Phases (Np threads per CTA):
@@ -508,7 +509,7 @@ __device__ __forceinline__ void agent_body(const AgentArgs& a, const int j0) {
                             residual_sums(first ? v0 : x0[i], w0, az, aw);
                             residual_sums(first ? v1 : x1[i], w1, az, aw);
                         }
-                        *reinterpret_cast<float4*>(uo + row * N + c) = make_float4(u0.x, u0.y, u1.x, u1.y);
+                        if (a.u) *reinterpret_cast<float4*>(uo + row * N + c) = make_float4(u0.x, u0.y, u1.x, u1.y);
                         *reinterpret_cast<float4*>(qp + row * N + c) = make_float4(q0.x, q0.y, q1.x, q1.y);
                     }
                 });

@@ -337,8 +337,10 @@ __device__ __forceinline__ void pair_body(const AgentArgs& a, const int j0, cons
     const bool first = a.first != 0;
     const bool res = a.residual != 0;
     const int row0 = rank * G::R;
-    const uint64_t pol_u = a.keep_u ? l2_policy_evict_last() : l2_policy_evict_normal();
+    const bool wu = a.u != nullptr;   // else the consensus gather reads q' next
+    const uint64_t pol_next = a.keep ? l2_policy_evict_last() : l2_policy_evict_normal();
     const uint64_t pol_first = l2_policy_evict_first();
+    const uint64_t pol_q = wu ? pol_first : pol_next;
     uint32_t parity = 0;
 
     // thread (k, b): first-stage butterfly b of slab row k, pixels (row0 + k, b + S1 t)
@@ -697,10 +699,12 @@ __device__ __forceinline__ void pair_body(const AgentArgs& a, const int j0, cons
                             acc_z = make_float2(az, bz);
                             acc_w = make_float2(aw, bw);
                         }
-                        st_l2_hint(u0 + s, ua, pol_u);      // read by the consensus gather next
-                        st_l2_hint(u1 + s, ub, pol_u);
-                        st_l2_hint(q0 + s, qn0, pol_first);  // read again only next iteration
-                        st_l2_hint(q1 + s, qn1, pol_first);
+                        if (wu) {
+                            st_l2_hint(u0 + s, ua, pol_next);
+                            st_l2_hint(u1 + s, ub, pol_next);
+                        }
+                        st_l2_hint(q0 + s, qn0, pol_q);
+                        st_l2_hint(q1 + s, qn1, pol_q);
                     }
                     // the next pair's values of these four pixels (the last
                     // pair of a run reloads its own, which keeps the loads

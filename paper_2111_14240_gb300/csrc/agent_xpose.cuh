@@ -290,8 +290,12 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
     const bool first = a.first != 0;
     const bool res = a.residual != 0;
     const int row0 = rank * G::R;
-    const uint64_t pol_u = a.keep_u ? l2_policy_evict_last() : l2_policy_evict_normal();
+    // the stack the consensus gather reads next (u where it is written, else
+    // q') may stay in L2; what is read again only next iteration is evict-first
+    const bool wu = a.u != nullptr;
+    const uint64_t pol_next = a.keep ? l2_policy_evict_last() : l2_policy_evict_normal();
     const uint64_t pol_first = l2_policy_evict_first();
+    const uint64_t pol_q = wu ? pol_first : pol_next;
     uint32_t parity = 0;
 
     // With one first-stage butterfly per thread (Np >= 128), a thread's 16
@@ -632,8 +636,8 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
                             const float2 w =
                                 agent_step2<kCheck>(x[h0 + t], v, dv[t], scale2, alpha2, inv1pa2, m2rho2, u, qn);
                             if constexpr (kRes) residual_sums(first ? v : xv[t], w, acc_z, acc_w);
-                            st_l2_hint(ur + s, u, pol_u);       // read by the consensus gather next
-                            st_l2_hint(qr + s, qn, pol_first);  // read again only next iteration
+                            if (wu) st_l2_hint(ur + s, u, pol_next);
+                            st_l2_hint(qr + s, qn, pol_q);
                         }
                     };
                     if (absent) pixels(std::true_type{});

@@ -1,10 +1,11 @@
-// L2 eviction-priority hints for the two streams that meet in L2 within one
-// iteration: the agent sweep writes u, which the consensus gather reads
-// right after, while q', the amplitudes and the stack reads of the sweep are
-// used once per iteration.  u is stored evict-last, the single-use streams
-// are marked evict-first, so more of u is still in L2 when the gather runs.
-// The evict-last hint is only given where u can mostly stay in L2 (a job's
-// u no larger than twice the L2), else u is stored evict-normal.
+// L2 eviction-priority hints for the stream that meets itself in L2 within
+// one iteration: the agent sweep writes q' (or u, consensus_from_q), which the
+// consensus gather reads right after, while the amplitudes and the stack
+// reads of the sweep are used once per iteration.  The stack the gather reads
+// is stored evict-last, the single-use streams are marked evict-first, so
+// more of it is still in L2 when the gather runs.  The evict-last hint is only
+// given where the stack can mostly stay in L2 (no larger than twice the L2),
+// else it is stored evict-normal.
 #pragma once
 
 #include <cstdint>

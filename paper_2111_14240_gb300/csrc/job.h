@@ -25,7 +25,7 @@ struct pmace_job {
     int cluster = 1;
     int variant = 0;
     int wpc = 1;              // windows per agent cluster
-    int keep_u = 0;           // u small enough to favour it in L2 for the gather
+    int keep = 0;             // stack small enough to favour it in L2 for the gather
     pmace::AgentPlanInfo plan{};
     int tiles_x = 0, tiles_y = 0, ntiles = 0;
     int tile_h = 16;          // gather tile height (rows), width kGatherTileW
@@ -35,7 +35,7 @@ struct pmace_job {
     int nslots = 0;           // scratch slots of split tiles
 
     float2 *q = nullptr, *u = nullptr, *xbar = nullptr, *probe = nullptr, *dinv = nullptr,
-           *tw = nullptr, *img_tmp = nullptr;
+           *tw = nullptr, *xhat = nullptr;
     void* y = nullptr;
     float *yscale = nullptr, *laminv = nullptr, *wk = nullptr;
     int2* offs = nullptr;
@@ -49,6 +49,7 @@ struct pmace_job {
 
     int64_t iterations = 0;
     float rho_pending = 0.5f;
+    bool xhat_valid = false;  // xhat holds x_hat of the current (q, xbar)
 
     std::vector<int32_t> offs_host;   // window corners, for rebuilding the overlap lists
 
@@ -70,5 +71,13 @@ namespace pmace {
 // Kernel arguments of one iteration of job h (pmace_api.cu).
 AgentArgs agent_args(const pmace_job* h, float alpha, float rho);
 GatherArgs gather_args(const pmace_job* h);
+// Arguments of one iteration's consensus gather (after agent_args with the
+// same rho).
+GatherArgs consensus_args(const pmace_job* h, float rho);
+// Whether the consensus of an iteration with this rho is taken from the
+// pending stack and the readout image instead of the stack u (consensus_args).
+bool consensus_from_q(float rho);
+// x_hat of the current state into h->xhat, unless it is there already.
+cudaError_t ensure_xhat(pmace_job* h, cudaStream_t s);
 
 }  // namespace pmace

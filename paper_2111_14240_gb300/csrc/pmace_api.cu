@@ -2,9 +2,11 @@
 //
 // A job keeps its whole working set resident on one GPU:
 //   q     [J][Np][Np] complex64  pending Mann stack q = v - 2 rho w
-//   u     [J][Np][Np] complex64  agent reflection u = 2w - v (input of G)
+//   u     [J][Np][Np] complex64  agent reflection u = 2w - v (input of G where
+//                                it is not taken from q), staging otherwise
 //   y     [J][Np][Np] f32 or f16 amplitudes, digit-reversed kernel order
 //   xbar  [n1][n2]    complex64  consensus image of the last iteration
+//   xhat  [n1][n2]    complex64  readout image x_hat of the state, where valid
 //   laminv[n1][n2]    f32        Lambda^-1 (0 where Lambda = 0)
 // plus the probe tables (d, 1/d, |d|^kappa, twiddles) and the scan-overlap
 // lists.  One iteration of Algorithm 1 is two launches: the fused agent
@@ -436,7 +438,7 @@ pmace_status build_tables(pmace_job* h, const std::vector<float>& probe_h,
 
 void free_job(pmace_job* h) {
     if (!h) return;
-    void* ptrs[] = {h->q, h->u, h->xbar, h->probe, h->dinv, h->tw, h->img_tmp, h->y, h->yscale,
+    void* ptrs[] = {h->q, h->u, h->xbar, h->probe, h->dinv, h->tw, h->y, h->yscale,
                     h->laminv, h->wk, h->offs, h->tile_list, h->units, h->tile_seg, h->gscratch,
                     h->gcounters, h->err, h->partials, h->red_out};
     for (void* p : ptrs)
@@ -519,8 +521,70 @@ AgentArgs agent_args(const pmace_job* h, float alpha, float rho) {
     a.wpc = h->wpc;
     a.err = h->err;
     a.residual = 1;
-    a.keep_u = h->keep_u;
+    a.keep = h->keep;
+    if (consensus_from_q(rho)) a.u = nullptr;
     return a;
+}
+
+// G(2w - v) without the stack u: u = 2w - v = (1/rho - 1) v - q'/rho with the
+// q' = v - 2 rho w that the sweep writes anyway, and Lambda^-1 sum_j P_j^t
+// |D|^kappa v_j is the readout image of the state before the iteration, so
+// the sweep writes one stack instead of two and the gather reads q' (8 bytes
+// a window pixel less, for 16 bytes an image pixel more; the readout of the
+// new state comes out of the same pass).  The factor 1/rho multiplies the
+// rounding of the average of q': up to 2 at rho >= 1/2, where the image is as
+// near to the 64-bit result as from u (rel-L2 after one iteration from a near
+// start 2.08e-7 against 2.06e-7 in a float32 emulation at rho 0.5, 2.09e-7
+// against 2.06e-7 at 0.6); at rho 0.4 it was 13 % further off and at 0.2
+// twice as far, so smaller rho keep u.
+bool consensus_from_q(float rho) { return rho >= 0.5f; }
+
+GatherArgs consensus_args(const pmace_job* h, float rho) {
+    GatherArgs g = gather_args(h);
+    g.out = h->xbar;
+    g.src = h->u;
+    if (consensus_from_q(rho)) {
+        g.src = h->q;
+        g.keep = h->keep;
+        g.xhat = h->xhat;
+        g.c1 = (float)(1.0 / (double)rho - 1.0);
+        g.c2 = (float)(1.0 / (double)rho);
+        g.two_rho = 2.0f * rho;
+    }
+    return g;
+}
+
+// Whether a caller is capturing `s` (the job's own capture_stream aside).
+static bool user_capture(const pmace_job* h, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    return cap == cudaStreamCaptureStatusActive && s != h->capture_stream;
+}
+
+// x_hat of the current state into dst.
+static cudaError_t readout(const pmace_job* h, float2* dst, cudaStream_t s) {
+    GatherArgs g = gather_args(h);
+    g.src = h->q;
+    g.xbar_in = h->xbar;
+    g.out = dst;
+    g.two_rho = 2.0f * h->rho_pending;
+    return launch_gather_readout(g, h->nunits, h->tile_h, s);
+}
+
+cudaError_t ensure_xhat(pmace_job* h, cudaStream_t s) {
+    // Under a caller's stream capture the readout is always recorded: the
+    // state may have been replaced by the time the graph is replayed.
+    const bool captured = user_capture(h, s);
+    if (h->xhat_valid && !captured) return cudaSuccess;
+    const cudaError_t e = readout(h, h->xhat, s);
+    if (e == cudaSuccess && !captured) h->xhat_valid = true;
+    return e;
+}
+
+// x_hat of the current state into device memory of the caller's.
+static cudaError_t readout_to(const pmace_job* h, float2* dst, cudaStream_t s) {
+    if (!h->xhat_valid || user_capture(h, s)) return readout(h, dst, s);
+    return launch_copy_image(dst, h->xhat, (int64_t)h->dims.n1 * h->dims.n2, s);
 }
 }  // namespace pmace
 
@@ -534,9 +598,9 @@ pmace_status launch_iteration(pmace_job* h, float alpha, float rho, cudaStream_t
     AgentArgs a = agent_args(h, alpha, rho);
     a.residual = residual ? 1 : 0;
     a.spectrum = spectrum;
-    GatherArgs g = gather_args(h);
-    g.src = h->u;
-    g.out = h->xbar;
+    const bool from_q = consensus_from_q(rho);
+    if (from_q) PM_CUDA(h, ensure_xhat(h, s));
+    const GatherArgs g = consensus_args(h, rho);
     if (events) PM_CUDA(h, record_pair(h->ev_agent, h->n_agent, true, s));
     PM_CUDA(h, agent_entry(h->dims.np, &a, h->variant, h->amp_f16, s, nullptr));
     if (events) {
@@ -545,6 +609,7 @@ pmace_status launch_iteration(pmace_job* h, float alpha, float rho, cudaStream_t
     }
     PM_CUDA(h, launch_gather_consensus(g, h->nunits, h->tile_h, s));
     if (events) PM_CUDA(h, record_pair(h->ev_cons, h->n_cons, false, s));
+    if (!from_q) h->xhat_valid = false;
     h->rho_pending = rho;
     h->iterations++;
     return PMACE_OK;
@@ -561,7 +626,9 @@ pmace_status ensure_graph(pmace_job* h, float alpha, float rho) {
     if (!h->capture_stream) PM_CUDA(h, cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
     const int64_t it_saved = h->iterations;
     const float rho_saved = h->rho_pending;
+    const bool xhat_saved = h->xhat_valid;
     h->iterations = std::max<int64_t>(it_saved, 1);
+    h->xhat_valid = true;   // made so before every replay
     h->rho_pending = rho;
     cudaGraph_t graph = nullptr;
     PM_CUDA(h, cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal));
@@ -571,6 +638,7 @@ pmace_status ensure_graph(pmace_job* h, float alpha, float rho) {
     cudaError_t e = cudaStreamEndCapture(h->capture_stream, &graph);
     h->iterations = it_saved;
     h->rho_pending = rho_saved;
+    h->xhat_valid = xhat_saved;
     if (st != PMACE_OK) {
         if (graph) cudaGraphDestroy(graph);
         return st;
@@ -703,7 +771,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
     {
         int l2 = 0;
         if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device) != cudaSuccess) cudaGetLastError();
-        h->keep_u = l2 > 0 && JP * sizeof(float2) <= 2 * (size_t)l2;
+        h->keep = l2 > 0 && JP * sizeof(float2) <= 2 * (size_t)l2;
     }
 
     auto bail = [&](pmace_status st) {
@@ -771,7 +839,10 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
     } while (0)
     PM_CREATE(dalloc(h, &h->q, JP));
     PM_CREATE(dalloc(h, &h->u, JP));
-    PM_CREATE(dalloc(h, &h->xbar, NI));
+    // both images in one allocation, the second on a 256-byte boundary
+    const size_t NIpad = (NI + 31) / 32 * 32;
+    PM_CREATE(dalloc(h, &h->xbar, NIpad + NI));
+    h->xhat = h->xbar + NIpad;
     PM_CREATE(dalloc(h, &h->laminv, NI));
     PM_CREATE(dalloc(h, &h->partials, (size_t)J * kMaxCluster * 4 + kPrepBlocks));
     PM_CREATE(dalloc(h, &h->red_out, (size_t)4));
@@ -880,7 +951,9 @@ pmace_status pmace_iterate(pmace_handle h, int32_t n, const pmace_step* step, vo
         pmace_status st = ensure_graph(h, alpha, rho);
         if (st != PMACE_OK) return st;
         for (; done + kGraphIters <= n - 1; done += kGraphIters) {
+            if (consensus_from_q(rho)) PM_CUDA(h, ensure_xhat(h, s));
             PM_CUDA(h, cudaGraphLaunch(h->graph, s));
+            if (!consensus_from_q(rho)) h->xhat_valid = false;
             h->iterations += kGraphIters;
         }
     }
@@ -920,6 +993,7 @@ pmace_status pmace_autotune(pmace_handle h, const pmace_step* step, int32_t iter
         if (r == cudaSuccess) r = cudaMemcpyAsync(h->xbar, x0, NI * sizeof(float2), cudaMemcpyDeviceToDevice, s);
         h->iterations = it0;
         h->rho_pending = rho0;
+        h->xhat_valid = false;
         return r;
     };
     // time `iters` iterations (after two untimed ones) of the current plan, ms per iteration
@@ -990,20 +1064,12 @@ pmace_status pmace_get_image(pmace_handle h, float* out, int out_on_device, void
     if (!out) return fail(h, PMACE_ERR_INVALID_ARG, "out is NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t NI = (size_t)h->dims.n1 * h->dims.n2;
-    float2* dst = reinterpret_cast<float2*>(out);
-    if (!out_on_device) {
-        if (!h->img_tmp) PM_CUDA(h, dalloc(h, &h->img_tmp, NI));
-        dst = h->img_tmp;
-    }
-    GatherArgs g = gather_args(h);
-    g.src = h->q;
-    g.xbar_in = h->xbar;
-    g.out = dst;
-    g.two_rho = 2.0f * h->rho_pending;
-    PM_CUDA(h, launch_gather_readout(g, h->nunits, h->tile_h, s));
-    if (!out_on_device) {
+    if (out_on_device) {
+        PM_CUDA(h, readout_to(h, reinterpret_cast<float2*>(out), s));
+    } else {
         int errflag = 0;
-        PM_CUDA(h, cudaMemcpyAsync(out, dst, NI * sizeof(float2), cudaMemcpyDeviceToHost, s));
+        PM_CUDA(h, ensure_xhat(h, s));   // there already after an iteration whose consensus came from q
+        PM_CUDA(h, cudaMemcpyAsync(out, h->xhat, NI * sizeof(float2), cudaMemcpyDeviceToHost, s));
         PM_CUDA(h, cudaMemcpyAsync(&errflag, h->err, sizeof(int), cudaMemcpyDeviceToHost, s));
         PM_CUDA(h, cudaStreamSynchronize(s));
         if (errflag & 2)
@@ -1110,6 +1176,7 @@ pmace_status pmace_set_state(pmace_handle h, const float* q, const float* xbar,
     if (!on_device) PM_CUDA(h, cudaStreamSynchronize(s));
     h->iterations = info->iterations;
     h->rho_pending = info->rho_pending;
+    h->xhat_valid = false;
     return PMACE_OK;
 }
 

@@ -33,7 +33,7 @@ constexpr int kErrBoundsBit = 8;
 struct AgentArgs {
     float2* q;              // [J][Np][Np] pending stack q = v - 2 rho w (read, then overwritten; the
                             // in-place variant keeps v there between its copy-in and copy-out)
-    float2* u;              // [J][Np][Np] written: u = 2w - v
+    float2* u;              // [J][Np][Np] written: u = 2w - v; NULL where the consensus is taken from q
     const float2* xbar;     // [n1][n2] consensus image of the previous iteration
     const void* y;          // [J][Np][Np] amplitudes in kernel (digit-reversed) order
     const float* yscale;    // [J] per-pattern scale (FP16 codes only)
@@ -48,7 +48,8 @@ struct AgentArgs {
     float alpha, rho_prev, rho_cur;
     int first;              // 1 on the first iteration of the job
     int residual;           // 1: write the residual partial sums (else they are left untouched)
-    int keep_u;             // 1: store u with the L2 evict-last hint (u fits about twice the L2)
+    int keep;               // 1: store the stack the gather reads next (q, or u where it is written) with the
+                            // L2 evict-last hint (the stack fits about twice the L2)
     int wpc;                // windows per cluster (transposing-exchange variant)
     int* err;               // bit 2: a bounded device-side wait gave up; bit 3: a bounds check of the
                             // PMACE_DEBUG build failed
@@ -69,9 +70,13 @@ struct GatherArgs {
     const float* laminv;    // [n1][n2] Lambda^-1 (0 where Lambda = 0)
     const float2* xbar_in;  // readout: consensus image
     float2* out;            // [n1][n2]
+    float2* xhat;           // consensus from q: [n1][n2] readout image of the state before the iteration, replaced by
+                            // that of the state after it; NULL: consensus from u
+    float c1, c2;           // consensus from q: 1 / rho - 1 and 1 / rho
+    int keep;               // 1: src is read again soon and may stay in L2 (else it is read evict-first)
     float* lam_out;         // weight-image mode: Lambda^-1 written here
     int n1, n2, np, tiles_x;
-    float two_rho;          // readout: 2 rho
+    float two_rho;          // readout, consensus from q: 2 rho
     // bounds of the tables, checked by the PMACE_DEBUG build (bit 3 of *err)
     int J, list_len, ntiles, nslots;
     int* err;
@@ -176,6 +181,8 @@ cudaError_t launch_init_stack(float2* q, const float2* init, float2 cval, const 
 cudaError_t launch_patches_from_state(const float2* q, const float2* xbar, const int2* offs,
                                       float2* v, int J, int np, int n1, int n2, float two_rho,
                                       int* err, cudaStream_t s);
+// dst = src, n complex values (8-byte aligned).
+cudaError_t launch_copy_image(float2* dst, const float2* src, int64_t n, cudaStream_t s);
 cudaError_t launch_check_finite(const float* data, int64_t n, int* err_flag, cudaStream_t s);
 // dst[j][e] = src[j][map[e]] for every window j and stored position e
 // (elem bytes per value: 2, 4 or 8).

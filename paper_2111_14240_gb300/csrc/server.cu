@@ -329,14 +329,14 @@ pmace_status pmace_server::tick() {
     std::vector<int2> gwork;
     for (int i : stepping) {
         const pmace_job* h = active[i].job;
-        GatherArgs g = gather_args(h);
-        g.src = h->u;
-        g.out = h->xbar;
         const int gd = (int)gdesc.size();
-        gdesc.push_back(g);
+        gdesc.push_back(consensus_args(h, active[i].req.step.rho));
         for (int t = 0; t < h->nunits; ++t) gwork.push_back(make_int2(gd, t));
     }
-    cudaError_t e = d_adesc.reserve(adesc.size());
+    cudaError_t e = cudaSuccess;
+    for (int i : stepping)   // a job's first tick: the readout image its consensus starts from
+        if (e == cudaSuccess && consensus_from_q(active[i].req.step.rho)) e = ensure_xhat(active[i].job, stream);
+    if (e == cudaSuccess) e = d_adesc.reserve(adesc.size());
     if (e == cudaSuccess) e = d_awork.reserve(awork.size());
     if (e == cudaSuccess) e = d_gdesc.reserve(gdesc.size());
     if (e == cudaSuccess) e = d_gwork.reserve(gwork.size());
@@ -362,6 +362,7 @@ pmace_status pmace_server::tick() {
         pmace_job* h = active[i].job;
         h->rho_pending = active[i].req.step.rho;
         h->iterations++;
+        if (!consensus_from_q(h->rho_pending)) h->xhat_valid = false;
     }
     ticks++;
     return PMACE_OK;

@@ -20,6 +20,11 @@ namespace pmace {
 // and needs no float atomics.
 //   MODE 0: Lambda = sum_i |d|^kappa (FP64), writes Lambda^-1 (0 where Lambda = 0)
 //   MODE 1: xbar = Lambda^-1 sum_i P_i^t |D|^kappa u_i                 (G, S6)
+//           or, with g.xhat, the same image from the stack q' = v - 2 rho w
+//           (u = 2w - v = (1/rho - 1) v - q' / rho, and the average of v is
+//           the readout image of the state before the iteration):
+//             xbar = (1/rho - 1) xhat - (1/rho) s,  s = Lambda^-1 sum_i P_i^t |D|^kappa q'_i,
+//             xhat = s + 2 rho xbar                (the readout of the new state)
 //   MODE 2: x_hat = Lambda^-1 sum_i P_i^t |D|^kappa q_i + 2 rho xbar   (readout)
 // A tile cut into several units: each unit stores its partial sums in its
 // scratch slot, fences, and counts itself in the tile's counter; the unit
@@ -52,7 +57,7 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
     const int np = g.np;
     const size_t P = (size_t)np * np;
 
-    const uint64_t pol_first = l2_policy_evict_first();   // u: this is its last read
+    const uint64_t pol_first = g.keep ? l2_policy_evict_normal() : l2_policy_evict_first();
     using Acc = typename std::conditional<MODE == 0, double, float2>::type;
     Acc acc[RPT];
 #pragma unroll
@@ -170,6 +175,16 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
         } else {
             const float li = __ldg(g.laminv + p);
             float2 v = make_float2(acc[r].x * li, acc[r].y * li);
+            if constexpr (MODE == 1) {
+                if (g.xhat) {
+                    const float2 xh = g.xhat[p];
+                    const float k = g.c2 * li;
+                    const float2 xb =
+                        make_float2(fmaf(-k, acc[r].x, g.c1 * xh.x), fmaf(-k, acc[r].y, g.c1 * xh.y));
+                    g.xhat[p] = make_float2(fmaf(g.two_rho, xb.x, v.x), fmaf(g.two_rho, xb.y, v.y));
+                    v = xb;
+                }
+            }
             if constexpr (MODE == 2) {
                 const float2 xb = __ldg(g.xbar_in + p);
                 v.x = fmaf(g.two_rho, xb.x, v.x);
@@ -391,6 +406,29 @@ cudaError_t launch_relayout_window(void* dst, const void* src, const int* map, i
                                                             map, J, np);
     else
         return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+// A copied image, in 16-byte pieces where both sides allow it.  A kernel and
+// not cudaMemcpyAsync: on a 200 x 200 image the call took longer on the host
+// than the launch of a kernel (a readout of image and patches after two
+// iterations 80 us against 73 us).
+__global__ void __launch_bounds__(256)
+copy_image_kernel(float2* __restrict__ dst, const float2* __restrict__ src, int64_t n, int wide) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    if (wide) {
+        for (int64_t i = t0; i < n / 2; i += step) reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
+        if (t0 == 0 && (n & 1)) dst[n - 1] = src[n - 1];
+    } else {
+        for (int64_t i = t0; i < n; i += step) dst[i] = src[i];
+    }
+}
+
+cudaError_t launch_copy_image(float2* dst, const float2* src, int64_t n, cudaStream_t s) {
+    const int wide = ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0;
+    const int64_t items = wide ? (n + 1) / 2 : n;
+    const int64_t blocks = (items + 255) / 256;
+    copy_image_kernel<<<(unsigned)(blocks < 1216 * 4 ? blocks : 1216 * 4), 256, 0, s>>>(dst, src, n, wide);
     return cudaGetLastError();
 }
 
