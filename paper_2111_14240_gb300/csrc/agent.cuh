@@ -81,8 +81,10 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // where A = 0; coefficients whose squared magnitude would underflow are
 // rescaled by 2^100 first.  With RES, also adds (y - |A|/Np)^2 and y^2 to
 // the residual sums; the returned value is the same either way.
+// The amplitudes come in units of `yunit`, and so does the result.
 template <bool RES = true>
-__device__ __forceinline__ float2 replace_magnitude(float2 xa, float y, float inv_n, float& acc_d, float& acc_y) {
+__device__ __forceinline__ float2 replace_magnitude(float2 xa, float y, float inv_n, float& acc_d, float& acc_y,
+                                                    float yunit = 1.0f) {
     float m2 = fmaf(xa.x, xa.x, xa.y * xa.y);
     float unscale = inv_n;
     if (m2 < 0x1p-100f) {
@@ -98,9 +100,9 @@ __device__ __forceinline__ float2 replace_magnitude(float2 xa, float y, float in
         o = xa * (y * rs);
     }
     if constexpr (RES) {
-        const float e = y - mag;
+        const float yu = y * yunit, e = yu - mag;
         acc_d = fmaf(e, e, acc_d);
-        acc_y = fmaf(y, y, acc_y);
+        acc_y = fmaf(yu, yu, acc_y);
     }
     return o;
 }
@@ -121,7 +123,7 @@ __device__ __forceinline__ float rsqrt_normal(float m) {
 // not finite) all R take the general path.
 template <bool RES, int R>
 __device__ __forceinline__ void replace_magnitudes(float2 (&x)[R], const float (&y)[R], float inv_n, float& acc_d,
-                                                   float& acc_y) {
+                                                   float& acc_y, float yunit = 1.0f) {
     float m2[R];
     bool general = false;
 #pragma unroll
@@ -131,16 +133,16 @@ __device__ __forceinline__ void replace_magnitudes(float2 (&x)[R], const float (
     }
     if (general) {
 #pragma unroll
-        for (int i = 0; i < R; ++i) x[i] = replace_magnitude<RES>(x[i], y[i], inv_n, acc_d, acc_y);
+        for (int i = 0; i < R; ++i) x[i] = replace_magnitude<RES>(x[i], y[i], inv_n, acc_d, acc_y, yunit);
         return;
     }
 #pragma unroll
     for (int i = 0; i < R; ++i) {
         const float rs = rsqrt_normal(m2[i]);
         if constexpr (RES) {
-            const float e = y[i] - m2[i] * rs * inv_n;
+            const float yu = y[i] * yunit, e = yu - m2[i] * rs * inv_n;
             acc_d = fmaf(e, e, acc_d);
-            acc_y = fmaf(y[i], y[i], acc_y);
+            acc_y = fmaf(yu, yu, acc_y);
         }
         x[i] = x[i] * (y[i] * rs);
     }
@@ -191,14 +193,20 @@ __device__ __forceinline__ float2 agent_step(float2 g, float2 v, float2 dv, floa
 // for a probe value treated as absent (dv = 0) at this pixel; without it
 // the caller knows there is none.
 __device__ __forceinline__ float2 mann_close2(float2 q, float2 xv, float2 trp2) { return __ffma2_rn(trp2, xv, q); }
+__device__ __forceinline__ float2 agent_w2(float2 g, float2 v, float2 dv, float2 scale2, float2 alpha2, float2 inv1pa2) {
+    return __fmul2_rn(__ffma2_rn(alpha2, v, cmul(dv, __fmul2_rn(g, scale2))), inv1pa2);
+}
+__device__ __forceinline__ float2 agent_u2(float2 v, float2 w) {
+    return __ffma2_rn(make_float2(2.f, 2.f), w, make_float2(-v.x, -v.y));
+}
 template <bool CHECK>
 __device__ __forceinline__ float2 agent_step2(float2 g, float2 v, float2 dv, float2 scale2, float2 alpha2,
                                               float2 inv1pa2, float2 m2rho2, float2& u, float2& qn) {
-    float2 w = __fmul2_rn(__ffma2_rn(alpha2, v, cmul(dv, __fmul2_rn(g, scale2))), inv1pa2);
+    float2 w = agent_w2(g, v, dv, scale2, alpha2, inv1pa2);
     if constexpr (CHECK) {
         if (dv.x == 0.f && dv.y == 0.f) w = v;
     }
-    u = __ffma2_rn(make_float2(2.f, 2.f), w, make_float2(-v.x, -v.y));
+    u = agent_u2(v, w);
     qn = __ffma2_rn(m2rho2, w, v);
     return w;
 }

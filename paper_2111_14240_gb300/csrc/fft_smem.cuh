@@ -269,9 +269,68 @@ struct Dft<16, INV> {
     }
 };
 
+// Radix 32 as 8 x 4 (j = 4 j1 + j2, k = k1 + 8 k2), the inner twiddles
+// W_32^(j2 k1) folded into the radix-4 pass as in radix 16: a factor is its
+// larger part (cosine or sine) times one whose parts are +-1 and the ratio
+// of the two (at most 1 in magnitude), which costs two fused multiply-adds;
+// the larger parts ride on the multiply-adds that take the place of the
+// radix-4 additions.
 template <bool INV>
 struct Dft<32, INV> {
-    __device__ __forceinline__ static void run(float2 (&x)[32]) { FourStep<8, 4, INV>::run(x); }
+    // a * W_32^m = scale<m>() * unscaled<m>(a)
+    template <int M>
+    __host__ __device__ static constexpr bool by_cos() {
+        const double c = k_cos32(M), s = k_sin32(M);
+        return c * c >= s * s;
+    }
+    template <int M>
+    __host__ __device__ static constexpr float scale() {
+        return (float)(by_cos<M>() ? k_cos32(M) : (INV ? k_sin32(M) : -k_sin32(M)));
+    }
+    template <int M>
+    __device__ __forceinline__ static float2 unscaled(float2 a) {
+        if constexpr (M % 32 == 0) {
+            return a;
+        } else if constexpr (by_cos<M>()) {   // cos (1 + i t)
+            constexpr float t = (float)((INV ? k_sin32(M) : -k_sin32(M)) / k_cos32(M));
+            return make_float2(fmaf(-t, a.y, a.x), fmaf(t, a.x, a.y));
+        } else {                              // sin (t + i)
+            constexpr float t = (float)(k_cos32(M) / (INV ? k_sin32(M) : -k_sin32(M)));
+            return make_float2(fmaf(t, a.x, -a.y), fmaf(t, a.y, a.x));
+        }
+    }
+    template <int K1>
+    __device__ __forceinline__ static void pass2(const float2 (&t)[4][8], float2 (&x)[32]) {
+        if constexpr (K1 == 0) {
+            float2 s[4] = {t[0][0], t[1][0], t[2][0], t[3][0]};
+            Dft<4, INV>::run(s);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) x[8 * k2] = s[k2];
+        } else {
+            const float2 u1 = unscaled<K1>(t[1][K1]), u2 = unscaled<2 * K1>(t[2][K1]), u3 = unscaled<3 * K1>(t[3][K1]);
+            constexpr float k1 = scale<K1>(), k2 = scale<2 * K1>();
+            constexpr float r = (float)((double)scale<3 * K1>() / (double)scale<K1>());
+            const float2 a = fma_real(k2, u2, t[0][K1]), b = fma_real(-k2, u2, t[0][K1]);
+            const float2 c = fma_real(r, u3, u1), e = fma_real(-r, u3, u1);
+            x[K1] = fma_real(k1, c, a);
+            x[K1 + 16] = fma_real(-k1, c, a);
+            // b -+ i k1 e
+            constexpr float g = INV ? k1 : -k1;
+            x[K1 + 8] = make_float2(fmaf(-g, e.y, b.x), fmaf(g, e.x, b.y));
+            x[K1 + 24] = make_float2(fmaf(g, e.y, b.x), fmaf(-g, e.x, b.y));
+        }
+        if constexpr (K1 < 7) pass2<K1 + 1>(t, x);
+    }
+    __device__ __forceinline__ static void run(float2 (&x)[32]) {
+        float2 t[4][8];
+#pragma unroll
+        for (int j2 = 0; j2 < 4; ++j2) {
+#pragma unroll
+            for (int j1 = 0; j1 < 8; ++j1) t[j2][j1] = x[4 * j1 + j2];
+            Dft<8, INV>::run(t[j2]);
+        }
+        pass2<0>(t, x);
+    }
 };
 
 // Padded shared-memory column index: one float2 of padding after every 16,

@@ -24,6 +24,7 @@ struct pmace_job {
     int amp_f16 = 0;
     int cluster = 1;
     int variant = 0;
+    int impl = 0;             // the kernel that runs it (agent_impl)
     int wpc = 1;              // windows per agent cluster
     int keep = 0;             // stack small enough to favour it in L2 for the gather
     pmace::AgentPlanInfo plan{};

@@ -140,8 +140,8 @@ std::vector<int> radices_of(int L) {
 // variants leave the column axis in column_order; the transposing exchange
 // runs the same two DIF stages along columns as along rows, so both axes end
 // in the DIF order.
-std::vector<int> amp_row_order(int np, int variant) {
-    const AgentVariant v = agent_variant_of(np, variant);
+std::vector<int> amp_row_order(int np, int impl) {
+    const AgentVariant v = agent_variant_of(np, impl);
     if (!v.exchange) return column_order(np, v.cluster);
     std::vector<int> perm;
     dif_order(radices_of(np), 0, np, perm);
@@ -159,10 +159,23 @@ std::vector<int> amp_row_order(int np, int variant) {
 // loads 512 contiguous bytes per instruction.  Value f of a thread (f = u r2
 // + i: butterfly u of the thread, element i) sits at kernel row
 // m r2 + i, column 16 rank + c, with m = (t + u threads) / 16 and
-// c = (t + u threads) % 16 (the column step's own indexing).
-std::vector<int> amp_layout(int np, int variant, int elem) {
-    const AgentVariant v = agent_variant_of(np, variant);
-    const std::vector<int> rows = amp_row_order(np, variant);
+// c = (t + u threads) % 16 (the column step's own indexing).  The register
+// sweep has a thread order of its own: value f = 16 b + i of thread
+// t = 32 w + 4 kr + kc is frequency row kr + 8 i, column kc + 4 (2 w + b).
+std::vector<int> amp_layout(int np, int impl, int elem) {
+    if (impl == kRegImpl) {
+        const int T = 512, CH = 16 / elem, NCH = 32 / CH;
+        std::vector<int> out((size_t)np * np);
+        for (int k = 0; k < NCH; ++k)
+            for (int t = 0; t < T; ++t)
+                for (int e = 0; e < CH; ++e) {
+                    const int f = k * CH + e, b = f / 16, i = f % 16, w = t / 32, kr = (t % 32) / 4, kc = t % 4;
+                    out[((size_t)k * T + t) * CH + e] = (kr + 8 * i) * np + kc + 4 * (2 * w + b);
+                }
+        return out;
+    }
+    const AgentVariant v = agent_variant_of(np, impl);
+    const std::vector<int> rows = amp_row_order(np, impl);
     std::vector<int> cols;
     dif_order(radices_of(np), 0, np, cols);
     std::vector<int> out((size_t)np * np);
@@ -194,14 +207,16 @@ std::vector<int> amp_layout(int np, int variant, int elem) {
 // barrier); on the 64009-window scan runs of 4, 8, 16 and 32 windows took
 // 8.27, 8.03, 7.93 and 7.92 ms (PMACE_AGENT_WPC fixes the run).
 // The packed-lane sweep counts in pairs of windows, so its runs are even.
-int windows_per_cluster(int np, int variant, int J, const AgentPlanInfo& info) {
-    const AgentVariant v = agent_variant_of(np, variant);
+// The register sweep, one CTA an SM, splits J evenly over the SMs.
+int windows_per_cluster(int np, int impl, int J, const AgentPlanInfo& info) {
+    const AgentVariant v = agent_variant_of(np, impl);
     if (!v.exchange) return v.windows;
     const int unit = v.exchange == 2 ? 2 : 1;   // the packed-lane sweep takes windows in pairs
     if (const char* env = std::getenv("PMACE_AGENT_WPC")) {   // fixed run length (rounded up to the unit)
         const int w = std::atoi(env);
         if (w > 0) return (w + unit - 1) / unit * unit;
     }
+    if (impl == kRegImpl) return (J + info.max_clusters - 1) / info.max_clusters;
     const int m = 4 * std::max(info.max_clusters, 1) * unit;
     return unit * std::max(1, std::min(16 / unit, (J + m - 1) / m));
 }
@@ -413,7 +428,7 @@ pmace_status build_tables(pmace_job* h, const std::vector<float>& probe_h,
     }
     // where the agent kernel reads each amplitude (spectrum orders of its
     // stages, and for the exchange variants the thread order)
-    const std::vector<int> layout = amp_layout(np, h->variant, h->amp_f16 ? 2 : 4);
+    const std::vector<int> layout = amp_layout(np, h->impl, h->amp_f16 ? 2 : 4);
 
     PM_CUDA(h, dalloc(h, &h->probe, P));
     PM_CUDA(h, dalloc(h, &h->dinv, P));
@@ -602,7 +617,7 @@ pmace_status launch_iteration(pmace_job* h, float alpha, float rho, cudaStream_t
     if (from_q) PM_CUDA(h, ensure_xhat(h, s));
     const GatherArgs g = consensus_args(h, rho);
     if (events) PM_CUDA(h, record_pair(h->ev_agent, h->n_agent, true, s));
-    PM_CUDA(h, agent_entry(h->dims.np, &a, h->variant, h->amp_f16, s, nullptr));
+    PM_CUDA(h, agent_entry(h->dims.np, &a, h->impl, h->amp_f16, s, nullptr));
     if (events) {
         PM_CUDA(h, record_pair(h->ev_agent, h->n_agent, false, s));
         PM_CUDA(h, record_pair(h->ev_cons, h->n_cons, true, s));
@@ -666,13 +681,14 @@ pmace_status switch_plan(pmace_job* h, int variant, int tile_h, cudaStream_t s) 
         return fail(h, PMACE_ERR_INVALID_ARG, "tile_h %d not in {8, 16, 32}", tile_h);
     if (variant != h->variant) {
         AgentPlanInfo info{};
-        if (agent_entry(np, nullptr, variant, h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
+        const int impl = agent_impl(np, variant, J);
+        if (agent_entry(np, nullptr, impl, h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
             cudaGetLastError();
             return fail(h, PMACE_ERR_UNSUPPORTED_SIZE, "agent variant %d cannot run on this device", variant);
         }
-        const int c_new = agent_variant_of(np, variant).cluster;
+        const int c_new = agent_variant_of(np, impl).cluster;
         const int elem = h->amp_f16 ? 2 : 4;
-        const std::vector<int> l_old = amp_layout(np, h->variant, elem), l_new = amp_layout(np, variant, elem);
+        const std::vector<int> l_old = amp_layout(np, h->impl, elem), l_new = amp_layout(np, impl, elem);
         if (l_old != l_new) {
             const size_t P = (size_t)np * np;
             std::vector<int> inv(P), map(P);
@@ -689,9 +705,10 @@ pmace_status switch_plan(pmace_job* h, int variant, int tile_h, cudaStream_t s) 
             if (e != cudaSuccess) return cuda_fail(h, e, "amplitude re-layout");
         }
         h->variant = variant;
+        h->impl = impl;
         h->cluster = c_new;
         h->plan = info;
-        h->wpc = windows_per_cluster(np, variant, J, info);
+        h->wpc = windows_per_cluster(np, impl, J, info);
     }
     if (tile_h != h->tile_h) {
         const pmace_status st = install_gather_tables(h, tile_h, s);
@@ -787,7 +804,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         for (int i = 0; i < kAgentVariants && chosen < 0; ++i) {
             const int v = (v0 + i) % kAgentVariants;
             AgentPlanInfo info{};
-            if (agent_entry(np, nullptr, v, h->amp_f16, s, &info) == cudaSuccess && info.launchable) {
+            if (agent_entry(np, nullptr, agent_impl(np, v, J), h->amp_f16, s, &info) == cudaSuccess && info.launchable) {
                 h->plan = info;
                 chosen = v;
             }
@@ -796,8 +813,9 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         if (chosen < 0)
             return bail(fail(h, PMACE_ERR_UNSUPPORTED_SIZE, "no launchable agent plan for np=%d", np));
         h->variant = chosen;
-        h->cluster = agent_variant_of(np, chosen).cluster;
-        h->wpc = windows_per_cluster(np, chosen, J, h->plan);
+        h->impl = agent_impl(np, chosen, J);
+        h->cluster = agent_variant_of(np, h->impl).cluster;
+        h->wpc = windows_per_cluster(np, h->impl, J, h->plan);
     }
     // gather tile height: PMACE_GATHER_TILE_H in {8, 16, 32}, default 16
     if (const char* env = std::getenv("PMACE_GATHER_TILE_H")) {
@@ -1023,7 +1041,7 @@ pmace_status pmace_autotune(pmace_handle h, const pmace_step* step, int32_t iter
     // agent variants at the current tile height, then tile heights for the best variant
     for (int v = 0; v < kAgentVariants && st == PMACE_OK; ++v) {
         AgentPlanInfo info{};
-        if (agent_entry(h->dims.np, nullptr, v, h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
+        if (agent_entry(h->dims.np, nullptr, agent_impl(h->dims.np, v, h->dims.J), h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
             cudaGetLastError();
             continue;
         }
@@ -1086,16 +1104,20 @@ pmace_status pmace_debug_spectra(pmace_handle h, const pmace_step* step, float* 
     if (!(step->alpha >= 0.f) || !std::isfinite(step->alpha) || !(step->rho > 0.f && step->rho < 1.f))
         return fail(h, PMACE_ERR_INVALID_ARG, "invalid step");
     const int np = h->dims.np, J = h->dims.J;
-    if (!agent_variant_of(np, h->variant).exchange)
+    if (!agent_variant_of(np, h->impl).exchange)
         return fail(h, PMACE_ERR_UNSUPPORTED_SIZE, "the spectrum check needs an exchange plan (variant %d is not)",
                     h->variant);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float2* dst = reinterpret_cast<float2*>(out);
     pmace_status st = launch_iteration(h, step->alpha, step->rho, s, false, true, dst);
     if (st != PMACE_OK) return st;
+    if (h->impl == kRegImpl) {   // written in natural order
+        PM_CUDA(h, cudaStreamSynchronize(s));
+        return PMACE_OK;
+    }
     // kernel order (row g, column c hold frequencies rows[g], cols[c]) to natural order, through u (dead now)
     const size_t P = (size_t)np * np;
-    std::vector<int> rows = amp_row_order(np, h->variant), cols, map(P);
+    std::vector<int> rows = amp_row_order(np, h->impl), cols, map(P);
     dif_order(radices_of(np), 0, np, cols);
     for (int g = 0; g < np; ++g)
         for (int c = 0; c < np; ++c) map[(size_t)rows[g] * np + cols[c]] = g * np + c;
@@ -1213,7 +1235,7 @@ pmace_status pmace_kernel_times(pmace_handle h, double* agent_ms, int64_t* agent
 pmace_status pmace_get_plan(pmace_handle h, pmace_plan* plan) {
     if (!h) return fail(nullptr, PMACE_ERR_INVALID_ARG, "NULL handle");
     if (!plan) return fail(h, PMACE_ERR_INVALID_ARG, "plan is NULL");
-    const AgentVariant v = agent_variant_of(h->dims.np, h->variant);
+    const AgentVariant v = agent_variant_of(h->dims.np, h->impl);
     plan->cluster = h->cluster;
     plan->threads = h->plan.threads;
     plan->smem_bytes = h->plan.smem_bytes;

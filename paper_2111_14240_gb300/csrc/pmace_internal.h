@@ -115,7 +115,11 @@ struct AgentVariant {
     int cluster, cols_per_thread, stage_y, windows, exchange;
 };
 constexpr int kAgentVariants = 6;
+// A second kernel behind a variant, not a variant of its own: the sweep that
+// holds whole windows in registers (agent_reg.cuh), one CTA a window.
+constexpr int kRegImpl = 6;
 __host__ __device__ constexpr AgentVariant agent_variant_of(int np, int v) {
+    if (v == kRegImpl) return {1, 1, 0, 1, 1};
     constexpr AgentVariant t32[kAgentVariants] = {
         {2, 1, 1, 1, 0}, {1, 1, 1, 1, 0}, {2, 1, 0, 2, 0}, {1, 1, 0, 1, 0}, {2, 1, 0, 1, 1}, {2, 1, 0, 2, 2}};
     constexpr AgentVariant t64[kAgentVariants] = {
@@ -135,6 +139,17 @@ __host__ __device__ constexpr AgentVariant agent_variant_of(int np, int v) {
 // windows).
 __host__ __device__ constexpr int default_agent_variant(int np, int J) {
     return np >= 64 ? 4 : J >= 1024 ? 1 : 0;
+}
+
+// The kernel that runs variant v for J windows of np x np.  The register
+// sweep takes a window an SM, the cluster sweep spreads one over eight CTAs,
+// which is the faster way while the windows do not fill the SMs: 128 x 128
+// windows, agent sweep in us, register against cluster: J = 36 21 / 16.6,
+// 64 21.3 / 20.7, 81 21.6 / 23.2, 120 22.3 / 29.7, 156 33.5 / 34.9, 342
+// 46 / 64, 900 91 / 125.
+constexpr int kReg128MinWindows = 72;
+__host__ __device__ constexpr int agent_impl(int np, int v, int J) {
+    return np == 128 && v == 4 && J >= kReg128MinWindows ? kRegImpl : v;
 }
 
 // Geometry of one agent plan (probe size, CTAs per patch).

@@ -289,14 +289,14 @@ pmace_status pmace_server::tick() {
         const int64_t rx = remaining(x), ry = remaining(y);
         return rx != ry ? rx < ry : active[x].req.id < active[y].req.id;
     });
-    // agent launches, one per (probe size, amplitude format, variant) group
+    // agent launches, one per (probe size, amplitude format, kernel) group
     std::map<std::tuple<int, int, int>, std::vector<int>> groups;
     int64_t px = 0;
     for (int i : cand) {
         Active& a = active[i];
         const pmace_job* h = a.job;
         if (px < tick_pixels || a.skipped >= kMaxSkippedTicks) {
-            groups[std::make_tuple(h->dims.np, h->amp_f16, h->variant)].push_back(i);
+            groups[std::make_tuple(h->dims.np, h->amp_f16, h->impl)].push_back(i);
             px += (int64_t)h->dims.J * h->dims.np * h->dims.np;
             a.skipped = 0;
         } else {
@@ -307,7 +307,7 @@ pmace_status pmace_server::tick() {
     std::vector<AgentArgs> adesc;
     std::vector<int2> awork;
     struct Launch {
-        int np, amp, variant, first_cluster, nclusters;
+        int np, amp, impl, first_cluster, nclusters;
     };
     std::vector<Launch> launches;
     std::vector<int> stepping;
@@ -351,7 +351,7 @@ pmace_status pmace_server::tick() {
         e = cudaMemcpyAsync(d_gwork.p, gwork.data(), gwork.size() * sizeof(int2), cudaMemcpyHostToDevice, stream);
     for (const Launch& L : launches) {
         if (e != cudaSuccess) break;
-        e = agent_batched(L.np, d_adesc.p, d_awork.p + L.first_cluster, L.nclusters, L.variant, L.amp, stream);
+        e = agent_batched(L.np, d_adesc.p, d_awork.p + L.first_cluster, L.nclusters, L.impl, L.amp, stream);
     }
     if (e == cudaSuccess) e = launch_gather_consensus_batched(d_gdesc.p, d_gwork.p, (int)gwork.size(), tile_h, stream);
     if (e != cudaSuccess) {
