@@ -246,6 +246,8 @@ def measured_peaks():
 
 def agent_kernel_name(plan) -> str:
     """The agent sweep kernel a plan launches."""
+    if plan.get("cluster") == 1 and plan.get("threads", 0) >= 128:
+        return "agent_reg32_kernel" if plan.get("threads") == 128 and plan.get("exchange") == 0 else "agent_reg_kernel"
     return {0: "agent_kernel", 1: "agent_xpose_kernel", 2: "agent_pair_kernel"}.get(plan.get("exchange"), "?")
 
 

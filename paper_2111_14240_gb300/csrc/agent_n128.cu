@@ -33,7 +33,7 @@ cudaError_t agent_entry_128(const AgentArgs* a, int v, int amp_f16, cudaStream_t
         case 3: return agent_variant<128, 8, 2, 0, 2>(a, amp_f16, s, info);
         case 4: return agent_xpose<128>(a, amp_f16, s, info);
         case 5: return agent_pair<128>(a, amp_f16, s, info);
-        case kRegImpl: return agent_reg128(a, amp_f16, s, info);
+        case kRegImpl: return agent_reg<128>(a, amp_f16, s, info);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -47,7 +47,7 @@ cudaError_t agent_entry_batched_128(const AgentArgs* descs, const int2* work, in
         case 3: return agent_variant_batched<128, 8, 2, 0, 2>(descs, work, nclusters, amp_f16, s);
         case 4: return agent_xpose_batched<128>(descs, work, nclusters, amp_f16, s);
         case 5: return agent_pair_batched<128>(descs, work, nclusters, amp_f16, s);
-        case kRegImpl: return agent_reg128_batched(descs, work, nclusters, amp_f16, s);
+        case kRegImpl: return agent_reg_batched<128>(descs, work, nclusters, amp_f16, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,6 +1,7 @@
 // Agent sweep instantiations for 64 x 64 probes (the variants of
 // agent_variant_of(64, .)).
 #include "agent.cuh"
+#include "agent_reg.cuh"
 #include "agent_xpose.cuh"
 
 namespace pmace {
@@ -28,6 +29,7 @@ cudaError_t agent_entry_64(const AgentArgs* a, int v, int amp_f16, cudaStream_t 
         case 2: return agent_variant<64, 2, 1, 1, 1>(a, amp_f16, s, info);
         case 3: return agent_variant<64, 4, 1, 0, 2>(a, amp_f16, s, info);
         case 4: return agent_xpose<64>(a, amp_f16, s, info);
+        case kRegImpl: return agent_reg<64>(a, amp_f16, s, info);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -40,6 +42,7 @@ cudaError_t agent_entry_batched_64(const AgentArgs* descs, const int2* work, int
         case 2: return agent_variant_batched<64, 2, 1, 1, 1>(descs, work, nclusters, amp_f16, s);
         case 3: return agent_variant_batched<64, 4, 1, 0, 2>(descs, work, nclusters, amp_f16, s);
         case 4: return agent_xpose_batched<64>(descs, work, nclusters, amp_f16, s);
+        case kRegImpl: return agent_reg_batched<64>(descs, work, nclusters, amp_f16, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -91,7 +91,7 @@ cudaError_t agent_entry(int np, const AgentArgs* a, int variant, int amp, cudaSt
 // agent_variant_of) when set and valid, else PMACE_AGENT_CLUSTER selects the
 // first variant with that cluster size, else the probe size's default
 // (default_agent_variant).
-int default_variant(int np, int J) {
+int default_variant(int np) {
     if (const char* env = std::getenv("PMACE_AGENT_PLAN")) {
         const int v = std::atoi(env);
         if (v >= 0 && v < kAgentVariants) return v;
@@ -101,7 +101,7 @@ int default_variant(int np, int J) {
         for (int v = 0; v < kAgentVariants; ++v)
             if (agent_variant_of(np, v).cluster == c) return v;
     }
-    return default_agent_variant(np, J);
+    return default_agent_variant(np);
 }
 
 // Row order of the amplitudes for a cluster size: kernel row g holds
@@ -160,17 +160,27 @@ std::vector<int> amp_row_order(int np, int impl) {
 // + i: butterfly u of the thread, element i) sits at kernel row
 // m r2 + i, column 16 rank + c, with m = (t + u threads) / 16 and
 // c = (t + u threads) % 16 (the column step's own indexing).  The register
-// sweep has a thread order of its own: value f = 16 b + i of thread
-// t = 32 w + 4 kr + kc is frequency row kr + 8 i, column kc + 4 (2 w + b).
+// sweep has a thread order of its own (agent_reg.cuh, chunk k of thread t at
+// (k threads + t) 16 bytes): value f = IR kb + i of thread t = 32 w + CC kr +
+// kc is frequency row kr + RR i, column kc + CC (KB w + kb).
 std::vector<int> amp_layout(int np, int impl, int elem) {
+    if (impl == kRegImpl && np == 32) {   // value f of lane kr is frequency row kr, column f
+        const int CH = 16 / elem;
+        std::vector<int> out((size_t)np * np);
+        for (int k = 0; k < 32 / CH; ++k)
+            for (int t = 0; t < 32; ++t)
+                for (int e = 0; e < CH; ++e) out[((size_t)k * 32 + t) * CH + e] = t * np + k * CH + e;
+        return out;
+    }
     if (impl == kRegImpl) {
-        const int T = 512, CH = 16 / elem, NCH = 32 / CH;
+        const int W = np * np / 1024, T = 32 * W, CC = np / 32, RR = np / W, IR = W, KB = 32 / IR;
+        const int CH = 16 / elem, NCH = 32 / CH;
         std::vector<int> out((size_t)np * np);
         for (int k = 0; k < NCH; ++k)
             for (int t = 0; t < T; ++t)
                 for (int e = 0; e < CH; ++e) {
-                    const int f = k * CH + e, b = f / 16, i = f % 16, w = t / 32, kr = (t % 32) / 4, kc = t % 4;
-                    out[((size_t)k * T + t) * CH + e] = (kr + 8 * i) * np + kc + 4 * (2 * w + b);
+                    const int f = k * CH + e, kb = f / IR, i = f % IR, w = t / 32, kr = (t % 32) / CC, kc = t % CC;
+                    out[((size_t)k * T + t) * CH + e] = (kr + RR * i) * np + kc + CC * (KB * w + kb);
                 }
         return out;
     }
@@ -207,9 +217,13 @@ std::vector<int> amp_layout(int np, int impl, int elem) {
 // barrier); on the 64009-window scan runs of 4, 8, 16 and 32 windows took
 // 8.27, 8.03, 7.93 and 7.92 ms (PMACE_AGENT_WPC fixes the run).
 // The packed-lane sweep counts in pairs of windows, so its runs are even.
-// The register sweep, one CTA an SM, splits J evenly over the SMs.
+// The register sweep splits J evenly over the CTAs the device holds.
 int windows_per_cluster(int np, int impl, int J, const AgentPlanInfo& info) {
     const AgentVariant v = agent_variant_of(np, impl);
+    if (impl == kRegImpl && np == 32) {   // four warps a CTA, a window each at a time
+        const int m = 4 * std::max(info.max_clusters, 1);
+        return 4 * std::max(1, (J + m - 1) / m);
+    }
     if (!v.exchange) return v.windows;
     const int unit = v.exchange == 2 ? 2 : 1;   // the packed-lane sweep takes windows in pairs
     if (const char* env = std::getenv("PMACE_AGENT_WPC")) {   // fixed run length (rounded up to the unit)
@@ -799,7 +813,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
 
     // plan: the requested variant if the device can run it, else the first that it can
     {
-        const int v0 = default_variant(np, J);
+        const int v0 = default_variant(np);
         int chosen = -1;
         for (int i = 0; i < kAgentVariants && chosen < 0; ++i) {
             const int v = (v0 + i) % kAgentVariants;

@@ -119,7 +119,7 @@ constexpr int kAgentVariants = 6;
 // holds whole windows in registers (agent_reg.cuh), one CTA a window.
 constexpr int kRegImpl = 6;
 __host__ __device__ constexpr AgentVariant agent_variant_of(int np, int v) {
-    if (v == kRegImpl) return {1, 1, 0, 1, 1};
+    if (v == kRegImpl) return np == 32 ? AgentVariant{1, 1, 0, 1, 0} : AgentVariant{1, 1, 0, 1, 1};
     constexpr AgentVariant t32[kAgentVariants] = {
         {2, 1, 1, 1, 0}, {1, 1, 1, 1, 0}, {2, 1, 0, 2, 0}, {1, 1, 0, 1, 0}, {2, 1, 0, 1, 1}, {2, 1, 0, 2, 2}};
     constexpr AgentVariant t64[kAgentVariants] = {
@@ -130,26 +130,26 @@ __host__ __device__ constexpr AgentVariant agent_variant_of(int np, int v) {
         {16, 2, 0, 1, 0}, {16, 2, 0, 2, 0}, {8, 1, 1, 1, 0}, {8, 2, 0, 1, 0}, {16, 1, 0, 1, 1}, {16, 1, 0, 2, 2}};
     return np == 32 ? t32[v] : np == 64 ? t64[v] : np == 128 ? t128[v] : t256[v];
 }
-// The fastest variant measured on GB300 for each probe size and J windows:
-// the transposing exchange (variant 4) for 64 x 64 and larger probes (on a
-// 1024^2 / 3600-window scan 0.174 ms against 0.179 ms for the best in-place
-// variant); for 32 x 32 probes one CTA per window (variant 1) once J fills
-// the GPU (0.042 ms against 0.066 ms on a 512^2 / 3600-window scan), else
-// two CTAs per window (variant 0: 0.0121 ms against 0.0140 ms for 169
-// windows).
-__host__ __device__ constexpr int default_agent_variant(int np, int J) {
-    return np >= 64 ? 4 : J >= 1024 ? 1 : 0;
-}
+// The fastest variant measured on GB300 for each probe size: variant 4 (the
+// register sweep or the transposing exchange, agent_impl) for 64 x 64 and
+// larger probes; for 32 x 32 probes variant 1, a window a warp (agent sweep in
+// us against variant 0, two CTAs a window: J = 1 10.3 / 10.8, 169 11.1 / 12.3,
+// 900 13 / 25, 3600 24 / 61).
+__host__ __device__ constexpr int default_agent_variant(int np) { return np >= 64 ? 4 : 1; }
 
 // The kernel that runs variant v for J windows of np x np.  The register
-// sweep takes a window an SM, the cluster sweep spreads one over eight CTAs,
-// which is the faster way while the windows do not fill the SMs: 128 x 128
-// windows, agent sweep in us, register against cluster: J = 36 21 / 16.6,
-// 64 21.3 / 20.7, 81 21.6 / 23.2, 120 22.3 / 29.7, 156 33.5 / 34.9, 342
-// 46 / 64, 900 91 / 125.
+// sweep takes a window a CTA (an SM for 128 x 128, a quarter of one for 64 x
+// 64), the cluster sweep spreads one over Np / 16 CTAs, which is the faster way
+// while the windows do not fill the SMs.  Agent sweep in us, register against
+// cluster, 128 x 128: J = 36 21 / 16.6, 64 21.3 / 20.7, 81 21.3 / 23.2, 120 22 /
+// 29.7, 342 46 / 64, 900 91 / 125; 64 x 64: J = 100 14.1 / 12.7, 168 15.2 / 14.6,
+// 374 19.3 / 24.9, 750 30 / 39, 3600 92 / 159.  The 32 x 32 register sweep (a
+// window a warp) takes the place of the in-place sweep with one CTA a window.
 constexpr int kReg128MinWindows = 72;
+constexpr int kReg64MinWindows = 180;
 __host__ __device__ constexpr int agent_impl(int np, int v, int J) {
-    return np == 128 && v == 4 && J >= kReg128MinWindows ? kRegImpl : v;
+    if (np == 32) return v == 1 ? kRegImpl : v;
+    return v == 4 && ((np == 128 && J >= kReg128MinWindows) || (np == 64 && J >= kReg64MinWindows)) ? kRegImpl : v;
 }
 
 // Geometry of one agent plan (probe size, CTAs per patch).
