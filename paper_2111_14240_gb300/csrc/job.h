@@ -44,7 +44,9 @@ struct pmace_job {
     int4* units = nullptr;
     int2* tile_seg = nullptr;
     float2* gscratch = nullptr;
-    int64_t gather_bytes = 0; // device bytes of the gather tables, included in `bytes`
+    char* mem = nullptr;        // the allocation the arrays above live in, but the gather's:
+    char* gather_mem = nullptr; // its tables and scratch (a plan switch replaces them)
+    int64_t gather_bytes = 0;   // device bytes of the gather tables, included in `bytes`
     double *partials = nullptr, *red_out = nullptr;
     int64_t bytes = 0;
 

@@ -26,6 +26,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace pmace;
@@ -66,13 +67,18 @@ pmace_status cuda_fail(pmace_job* h, cudaError_t e, const char* what) {
         if (e_ != cudaSuccess) return cuda_fail((h), e_, #call);    \
     } while (0)
 
-template <typename T>
-cudaError_t dalloc(pmace_job* h, T** p, size_t count) {
-    const size_t bytes = std::max<size_t>(count * sizeof(T), 16);
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
-    if (e == cudaSuccess) h->bytes += (int64_t)bytes;
-    return e;
-}
+// Arrays laid out one after another in one allocation, each on a 256-byte
+// boundary: a job made of some twenty cudaMalloc and cudaFree calls spent
+// about 1 ms in them (31 us and 15-90 us a call).
+struct Layout {
+    size_t bytes = 0;
+    template <typename T>
+    size_t add(size_t count) {
+        const size_t at = bytes;
+        bytes += (std::max<size_t>(count * sizeof(T), 16) + 255) / 256 * 256;
+        return at;
+    }
+};
 
 bool np_supported(int np) { return np == 32 || np == 64 || np == 128 || np == 256; }
 
@@ -174,14 +180,14 @@ std::vector<int> amp_layout(int np, int impl, int elem) {
     }
     if (impl == kRegImpl) {
         const int W = np * np / 1024, T = 32 * W, CC = np / 32, RR = np / W, IR = W, KB = 32 / IR;
-        const int CH = 16 / elem, NCH = 32 / CH;
+        const int sh = elem == 2 ? 3 : 2, CH = 1 << sh;   // 16-byte chunks
         std::vector<int> out((size_t)np * np);
-        for (int k = 0; k < NCH; ++k)
-            for (int t = 0; t < T; ++t)
-                for (int e = 0; e < CH; ++e) {
-                    const int f = k * CH + e, kb = f / IR, i = f % IR, w = t / 32, kr = (t % 32) / CC, kc = t % CC;
-                    out[((size_t)k * T + t) * CH + e] = (kr + RR * i) * np + kc + CC * (KB * w + kb);
-                }
+        for (int w = 0, t = 0; w < W; ++w)
+            for (int kr = 0; kr < RR; ++kr)
+                for (int kc = 0; kc < CC; ++kc, ++t)
+                    for (int kb = 0, f = 0; kb < KB; ++kb)
+                        for (int i = 0; i < IR; ++i, ++f)
+                            out[((size_t)(f >> sh) * T + t) * CH + (f & (CH - 1))] = (kr + RR * i) * np + kc + CC * (KB * w + kb);
         return out;
     }
     const AgentVariant v = agent_variant_of(np, impl);
@@ -281,11 +287,22 @@ void overlap_lists(const pmace_dims& d, const std::vector<int32_t>& offs_h, Gath
 }
 
 // Units of the tables' lists for block length B (empty tiles keep one unit).
-int64_t count_units(const GatherTables& t, int B) {
+// `quot` is scratch: i / B of every window i, filled without divisions.
+int64_t count_units(const GatherTables& t, int B, int J, std::vector<int>& quot) {
+    quot.resize(J);
+    for (int i = 0, q = 0; i < J; ++q)
+        for (int k = 0; k < B && i < J; ++k) quot[i++] = q;
     int64_t n = 0;
     for (int k = 0; k < t.ntiles; ++k) {
         int64_t runs = 1;
-        for (int a = t.cnt[k] + 1; a < t.cnt[k + 1]; ++a) runs += t.list[a] / B != t.list[a - 1] / B;
+        if (t.cnt[k] < t.cnt[k + 1]) {
+            int last = quot[t.list[t.cnt[k]]];
+            for (int a = t.cnt[k] + 1; a < t.cnt[k + 1]; ++a) {
+                const int q = quot[t.list[a]];
+                runs += q != last;
+                last = q;
+            }
+        }
         n += runs;
     }
     return n;
@@ -329,10 +346,8 @@ constexpr int64_t kGatherMinWindows = 16;
 // kGatherMinWindows)) units (PMACE_GATHER_UNITS and PMACE_GATHER_SEG, if
 // set, replace the two constants); J when the image alone has that many
 // tiles.  A function of the job's scan alone.
-int gather_block_length(const pmace_dims& d, const std::vector<int32_t>& offs_h) {
-    GatherTables t;
-    t.tile_h = 16;
-    overlap_lists(d, offs_h, t);
+// `t`: the overlap lists of the 16-row tiles.
+int gather_block_length(const pmace_dims& d, const GatherTables& t) {
     int64_t minw = kGatherMinWindows, units = kGatherTargetUnits;
     if (const char* env = std::getenv("PMACE_GATHER_SEG")) {
         const int v = std::atoi(env);
@@ -345,65 +360,63 @@ int gather_block_length(const pmace_dims& d, const std::vector<int32_t>& offs_h)
     const int64_t total = t.cnt[t.ntiles];
     const int64_t target = std::max<int64_t>(t.ntiles, std::min<int64_t>(units, total / minw));
     if (t.ntiles >= target) return std::max(d.J, 1);
+    std::vector<int> quot;
     int lo = 1, hi = std::max(d.J, 1);   // count_units(hi) = ntiles <= target
     while (lo < hi) {
         const int mid = lo + (hi - lo) / 2;
-        if (count_units(t, mid) <= target) hi = mid;
+        if (count_units(t, mid, d.J, quot) <= target) hi = mid;
         else lo = mid + 1;
     }
     return lo;
 }
 
-GatherTables make_gather_tables(const pmace_dims& d, const std::vector<int32_t>& offs_h, int tile_h, int B) {
-    GatherTables t;
-    t.tile_h = tile_h;
-    overlap_lists(d, offs_h, t);
-    cut_units(t, B);
-    return t;
-}
-
 // Build the gather tables for tile height tile_h, upload them, and replace
-// the job's current ones (freed after `s` has been synchronised).
-pmace_status install_gather_tables(pmace_job* h, int tile_h, cudaStream_t s) {
-    if (h->gblock <= 0) h->gblock = gather_block_length(h->dims, h->offs_host);
-    const GatherTables t = make_gather_tables(h->dims, h->offs_host, tile_h, h->gblock);
-    int* list = nullptr;
-    int4* units = nullptr;
-    int2* seg = nullptr;
-    float2* scratch = nullptr;
-    int* counters = nullptr;
-    const size_t slot = (size_t)tile_h * kGatherTileW;
-    const size_t b_list = t.list.size() * sizeof(int), b_units = t.units.size() * sizeof(int4),
-                 b_seg = t.seg.size() * sizeof(int2),
-                 b_scr = std::max<size_t>((size_t)t.nslots * slot, 1) * sizeof(float2),
-                 b_cnt = (size_t)t.ntiles * sizeof(int);
-    cudaError_t e = cudaMalloc(&list, b_list);
-    if (e == cudaSuccess) e = cudaMalloc(&units, b_units);
-    if (e == cudaSuccess) e = cudaMalloc(&seg, b_seg);
-    if (e == cudaSuccess) e = cudaMalloc(&scratch, b_scr);
-    if (e == cudaSuccess) e = cudaMalloc(&counters, b_cnt);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(list, t.list.data(), b_list, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(units, t.units.data(), b_units, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(seg, t.seg.data(), b_seg, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counters, 0, b_cnt, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host tables die on return
+// the job's current ones (freed after `s` has been synchronised).  `staged`,
+// where given, keeps the host copy until the caller has synchronised `s`;
+// without it the call does.
+pmace_status install_gather_tables(pmace_job* h, int tile_h, cudaStream_t s, std::vector<char>* staged = nullptr) {
+    GatherTables t;
+    t.tile_h = 16;
+    if (h->gblock <= 0) {
+        overlap_lists(h->dims, h->offs_host, t);
+        h->gblock = gather_block_length(h->dims, t);
+    }
+    if (t.cnt.empty() || tile_h != 16) {
+        t.tile_h = tile_h;
+        overlap_lists(h->dims, h->offs_host, t);
+    }
+    cut_units(t, h->gblock);
+    Layout lay;   // the tables, then the scratch slots, which need no upload
+    const size_t o_units = lay.add<int4>(t.units.size()), o_seg = lay.add<int2>(t.seg.size()),
+                 o_cnt = lay.add<int>(t.ntiles), o_list = lay.add<int>(t.list.size()), up = lay.bytes,
+                 o_scr = lay.add<float2>(std::max<size_t>((size_t)t.nslots * tile_h * kGatherTileW, 1));
+    std::vector<char> own;
+    std::vector<char>& host = staged ? *staged : own;
+    host.assign(up, 0);   // the tile counters start at 0
+    std::memcpy(host.data() + o_units, t.units.data(), t.units.size() * sizeof(int4));
+    std::memcpy(host.data() + o_seg, t.seg.data(), t.seg.size() * sizeof(int2));
+    std::memcpy(host.data() + o_list, t.list.data(), t.list.size() * sizeof(int));
+    char* mem = nullptr;
+    cudaError_t e = cudaMalloc(&mem, lay.bytes);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(mem, host.data(), up, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && !staged) e = cudaStreamSynchronize(s);   // the host copy dies on return
     if (e != cudaSuccess) {
-        for (void* p : {(void*)list, (void*)units, (void*)seg, (void*)scratch, (void*)counters})
-            if (p) cudaFree(p);
+        if (mem) {
+            cudaStreamSynchronize(s);
+            cudaFree(mem);
+        }
         return cuda_fail(h, e, "gather tables");
     }
-    for (void* p : {(void*)h->tile_list, (void*)h->units, (void*)h->tile_seg, (void*)h->gscratch,
-                    (void*)h->gcounters})
-        if (p) cudaFree(p);
-    const int64_t bytes = (int64_t)(b_list + b_units + b_seg + b_scr + b_cnt);
-    h->bytes += bytes - h->gather_bytes;
-    h->gather_bytes = bytes;
-    h->tile_list = list;
+    if (h->gather_mem) cudaFree(h->gather_mem);
+    h->bytes += (int64_t)lay.bytes - h->gather_bytes;
+    h->gather_bytes = (int64_t)lay.bytes;
+    h->gather_mem = mem;
+    h->tile_list = reinterpret_cast<int*>(mem + o_list);
     h->list_len = (int)t.list.size();
-    h->units = units;
-    h->tile_seg = seg;
-    h->gscratch = scratch;
-    h->gcounters = counters;
+    h->units = reinterpret_cast<int4*>(mem + o_units);
+    h->tile_seg = reinterpret_cast<int2*>(mem + o_seg);
+    h->gscratch = reinterpret_cast<float2*>(mem + o_scr);
+    h->gcounters = reinterpret_cast<int*>(mem + o_cnt);
     h->tile_h = t.tile_h;
     h->tiles_x = t.tiles_x;
     h->tiles_y = t.tiles_y;
@@ -413,29 +426,19 @@ pmace_status install_gather_tables(pmace_job* h, int tile_h, cudaStream_t s) {
     return PMACE_OK;
 }
 
-pmace_status build_tables(pmace_job* h, const std::vector<float>& probe_h,
-                          const std::vector<int32_t>& offs_h, cudaStream_t s,
-                          std::vector<std::vector<char>>& keep, int** perm_out) {
+// The probe tables (d as given, 1/d and |d|^kappa by a kernel, in double),
+// the twiddles, the window corners and the amplitude layout, on their way to
+// the device; `keep` holds the host sources until `s` is synchronised.
+pmace_status build_tables(pmace_job* h, const std::vector<float>& probe_h, int* layout_d, cudaStream_t s,
+                          std::vector<std::vector<char>>& keep) {
     const int np = h->dims.np, J = h->dims.J;
     const size_t P = (size_t)np * np;
-    // probe tables in double, rounded once
-    std::vector<float2> d(P), dinv(P), tw(np);
-    std::vector<float> wk(P);
-    double amax = 0.0;
-    for (size_t i = 0; i < P; ++i)
-        amax = std::max(amax, std::hypot((double)probe_h[2 * i], (double)probe_h[2 * i + 1]));
+    double m2max = 0.0;
     for (size_t i = 0; i < P; ++i) {
         const double re = probe_h[2 * i], im = probe_h[2 * i + 1];
-        const double m = std::hypot(re, im);
-        d[i] = make_float2((float)re, (float)im);
-        wk[i] = (float)std::pow(m, (double)h->dims.kappa);
-        if (m > 1e-30 * amax && m > 0.0) {
-            const double m2 = re * re + im * im;
-            dinv[i] = make_float2((float)(re / m2), (float)(-im / m2));
-        } else {
-            dinv[i] = make_float2(0.f, 0.f);
-        }
+        m2max = std::max(m2max, re * re + im * im);
     }
+    std::vector<float2> tw(np);
     for (int m = 0; m < np; ++m) {
         const double ang = -2.0 * M_PI * (double)m / (double)np;
         tw[m] = make_float2((float)std::cos(ang), (float)std::sin(ang));
@@ -443,35 +446,23 @@ pmace_status build_tables(pmace_job* h, const std::vector<float>& probe_h,
     // where the agent kernel reads each amplitude (spectrum orders of its
     // stages, and for the exchange variants the thread order)
     const std::vector<int> layout = amp_layout(np, h->impl, h->amp_f16 ? 2 : 4);
-
-    PM_CUDA(h, dalloc(h, &h->probe, P));
-    PM_CUDA(h, dalloc(h, &h->dinv, P));
-    PM_CUDA(h, dalloc(h, &h->tw, (size_t)np));
-    PM_CUDA(h, dalloc(h, &h->wk, P));
-    PM_CUDA(h, dalloc(h, &h->offs, (size_t)J));
     auto up = [&](void* dst, const void* src, size_t bytes) -> cudaError_t {
         keep.emplace_back((const char*)src, (const char*)src + bytes);   // alive until the sync
         return cudaMemcpyAsync(dst, keep.back().data(), bytes, cudaMemcpyHostToDevice, s);
     };
-    PM_CUDA(h, up(h->probe, d.data(), P * sizeof(float2)));
-    PM_CUDA(h, up(h->dinv, dinv.data(), P * sizeof(float2)));
+    PM_CUDA(h, cudaMemcpyAsync(h->probe, probe_h.data(), P * sizeof(float2), cudaMemcpyHostToDevice, s));
+    PM_CUDA(h, launch_probe_tables(h->probe, h->dinv, h->wk, (int)P, (double)h->dims.kappa, 1e-30 * std::sqrt(m2max), s));
     PM_CUDA(h, up(h->tw, tw.data(), np * sizeof(float2)));
-    PM_CUDA(h, up(h->wk, wk.data(), P * sizeof(float)));
-    PM_CUDA(h, up(h->offs, offs_h.data(), (size_t)J * 2 * sizeof(int32_t)));
-    // the layout table lives only until the amplitude pass
-    PM_CUDA(h, cudaMalloc(perm_out, P * sizeof(int)));
-    PM_CUDA(h, up(*perm_out, layout.data(), P * sizeof(int)));
+    PM_CUDA(h, cudaMemcpyAsync(h->offs, h->offs_host.data(), (size_t)J * 2 * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    PM_CUDA(h, up(layout_d, layout.data(), P * sizeof(int)));
     return PMACE_OK;
 }
 
 
 void free_job(pmace_job* h) {
     if (!h) return;
-    void* ptrs[] = {h->q, h->u, h->xbar, h->probe, h->dinv, h->tw, h->y, h->yscale,
-                    h->laminv, h->wk, h->offs, h->tile_list, h->units, h->tile_seg, h->gscratch,
-                    h->gcounters, h->err, h->partials, h->red_out};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    if (h->mem) cudaFree(h->mem);
+    if (h->gather_mem) cudaFree(h->gather_mem);
     for (auto* v : {&h->ev_agent, &h->ev_cons})
         for (auto& e : *v) {
             if (e.a) cudaEventDestroy(e.a);
@@ -839,8 +830,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
 
     // host copies of the small inputs
     std::vector<float> probe_h(2 * P);
-    std::vector<int32_t> offs_h(offsets, offsets + 2 * (size_t)J);
-    h->offs_host = offs_h;
+    h->offs_host.assign(offsets, offsets + 2 * (size_t)J);
     if (const char* env = std::getenv("PMACE_GRAPHS")) h->use_graphs = std::atoi(env) != 0;
     if (inputs_on_device) {
         cudaError_t e = cudaMemcpy(probe_h.data(), probe, 2 * P * sizeof(float), cudaMemcpyDeviceToHost);
@@ -851,38 +841,56 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
     for (float v : probe_h)
         if (!std::isfinite(v)) return bail(fail(h, PMACE_ERR_INVALID_ARG, "probe has non-finite values"));
 
+    // host sources of the uploads below; every way out synchronises `s` first
     std::vector<std::vector<char>> keep;
     keep.reserve(16);
-    int* perm_d = nullptr;
-    auto bail_perm = [&](pmace_status st2) {
+    std::vector<char> staged;
+    auto bail_sync = [&](pmace_status st2) {
         cudaStreamSynchronize(s);
-        if (perm_d) cudaFree(perm_d);
         return bail(st2);
     };
-    pmace_status st = build_tables(h, probe_h, offs_h, s, keep, &perm_d);
-    if (st == PMACE_OK) st = install_gather_tables(h, h->tile_h, s);
-    if (st != PMACE_OK) return bail_perm(st);
 
     cudaError_t e;
 #define PM_CREATE(call)                                                    \
     do {                                                                   \
         e = (call);                                                        \
-        if (e != cudaSuccess) return bail_perm(cuda_fail(h, e, #call));   \
+        if (e != cudaSuccess) return bail_sync(cuda_fail(h, e, #call));   \
     } while (0)
-    PM_CREATE(dalloc(h, &h->q, JP));
-    PM_CREATE(dalloc(h, &h->u, JP));
-    // both images in one allocation, the second on a 256-byte boundary
-    const size_t NIpad = (NI + 31) / 32 * 32;
-    PM_CREATE(dalloc(h, &h->xbar, NIpad + NI));
-    h->xhat = h->xbar + NIpad;
-    PM_CREATE(dalloc(h, &h->laminv, NI));
-    PM_CREATE(dalloc(h, &h->partials, (size_t)J * kMaxCluster * 4 + kPrepBlocks));
-    PM_CREATE(dalloc(h, &h->red_out, (size_t)4));
-    PM_CREATE(dalloc(h, &h->err, (size_t)1));
-    PM_CREATE(cudaMemsetAsync(h->err, 0, sizeof(int), s));
     const size_t ybytes = JP * (h->amp_f16 ? sizeof(__half) : sizeof(float));
-    PM_CREATE(cudaMalloc(&h->y, std::max<size_t>(ybytes, 16)));
-    h->bytes += (int64_t)ybytes;
+    int* layout_d = nullptr;   // the amplitude layout, used by the amplitude pass only
+    {
+        Layout lay;
+        const size_t o_q = lay.add<float2>(JP), o_u = lay.add<float2>(JP), o_y = lay.add<char>(ybytes),
+                     o_xbar = lay.add<float2>(NI), o_xhat = lay.add<float2>(NI), o_lam = lay.add<float>(NI),
+                     o_probe = lay.add<float2>(P), o_dinv = lay.add<float2>(P), o_wk = lay.add<float>(P),
+                     o_layout = lay.add<int>(P), o_tw = lay.add<float2>(np), o_offs = lay.add<int2>(J),
+                     o_scale = lay.add<float>(h->amp_f16 ? J : 0),
+                     o_part = lay.add<double>((size_t)J * kMaxCluster * 4 + kPrepBlocks), o_red = lay.add<double>(4),
+                     o_err = lay.add<int>(1);
+        PM_CREATE(cudaMalloc(&h->mem, lay.bytes));
+        h->bytes = (int64_t)lay.bytes;
+        auto at = [&](size_t o, auto*& p) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(h->mem + o); };
+        at(o_q, h->q);
+        at(o_u, h->u);
+        h->y = h->mem + o_y;
+        at(o_xbar, h->xbar);
+        at(o_xhat, h->xhat);
+        at(o_lam, h->laminv);
+        at(o_probe, h->probe);
+        at(o_dinv, h->dinv);
+        at(o_wk, h->wk);
+        at(o_layout, layout_d);
+        at(o_tw, h->tw);
+        at(o_offs, h->offs);
+        if (h->amp_f16) at(o_scale, h->yscale);
+        at(o_part, h->partials);
+        at(o_red, h->red_out);
+        at(o_err, h->err);
+    }
+    pmace_status st = build_tables(h, probe_h, layout_d, s, keep);
+    if (st == PMACE_OK) st = install_gather_tables(h, h->tile_h, s, &staged);
+    if (st != PMACE_OK) return bail_sync(st);
+    PM_CREATE(cudaMemsetAsync(h->err, 0, sizeof(int), s));
 
     // amplitudes to kernel order (staged through u when they come from the host)
     const void* amps_dev = amps;
@@ -890,13 +898,11 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         PM_CREATE(cudaMemcpyAsync(h->u, amps, ybytes, cudaMemcpyHostToDevice, s));
         amps_dev = h->u;
     }
-    if (h->amp_f16) {
-        PM_CREATE(dalloc(h, &h->yscale, (size_t)J));
+    if (h->amp_f16)
         PM_CREATE(cudaMemcpyAsync(h->yscale, scales, J * sizeof(float),
                                   inputs_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-    }
     double* sum_partials = h->partials + (size_t)J * kMaxCluster * 4;
-    PM_CREATE(launch_prep_amps(amps_dev, h->amp_f16, h->yscale, h->y, perm_d, J, np,
+    PM_CREATE(launch_prep_amps(amps_dev, h->amp_f16, h->yscale, h->y, layout_d, J, np,
                                sum_partials, h->err, kPrepBlocks, s));
     PM_CREATE(launch_reduce_partials(sum_partials, kPrepBlocks, 1, h->red_out, s));
 
@@ -905,16 +911,10 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
     g.lam_out = h->laminv;
     PM_CREATE(launch_gather_weights(g, h->nunits, h->tile_h, s));
 
-    // initial stacks
-    double sumsq = 0.0;
-    PM_CREATE(cudaMemcpyAsync(&sumsq, h->red_out, sizeof(double), cudaMemcpyDeviceToHost, s));
-    PM_CREATE(cudaStreamSynchronize(s));
-    int errflag = 0;
-    PM_CREATE(cudaMemcpy(&errflag, h->err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (errflag & 1) return bail_perm(fail(h, PMACE_ERR_INVALID_ARG, "amplitudes must be finite and >= 0"));
+    // initial stacks (without init: the constant sqrt(sum y^2 / (J ||d||^2)),
+    // taken from the sum on the device)
     double dsq = 0.0;
     for (size_t i = 0; i < 2 * P; ++i) dsq += (double)probe_h[i] * probe_h[i];
-    const float cval = (dsq > 0.0) ? (float)std::sqrt(sumsq / ((double)J * dsq)) : 0.f;
     const float2* init_dev = nullptr;
     if (init) {
         if (inputs_on_device) {
@@ -925,11 +925,13 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         }
         PM_CREATE(launch_check_finite(reinterpret_cast<const float*>(init_dev), (int64_t)NI * 2, h->err, s));
     }
-    PM_CREATE(launch_init_stack(h->q, init_dev, make_float2(cval, 0.f), h->offs, J, np, D.n2, s));
+    PM_CREATE(launch_init_stack(h->q, init_dev, h->red_out, (double)J * dsq, h->offs, J, np, D.n2, s));
     PM_CREATE(cudaMemsetAsync(h->xbar, 0, NI * sizeof(float2), s));
+    int errflag = 0;
+    PM_CREATE(cudaMemcpyAsync(&errflag, h->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     PM_CREATE(cudaStreamSynchronize(s));
-    PM_CREATE(cudaMemcpy(&errflag, h->err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (errflag & 2) return bail_perm(fail(h, PMACE_ERR_INVALID_ARG, "init has non-finite values"));
+    if (errflag & 1) return bail(fail(h, PMACE_ERR_INVALID_ARG, "amplitudes must be finite and >= 0"));
+    if (errflag & 2) return bail(fail(h, PMACE_ERR_INVALID_ARG, "init has non-finite values"));
     // Host-side fault injection for the tests of the error paths:
     // PMACE_INJECT_WAIT_TIMEOUT=1 marks the new job as if a bounded exchange
     // wait of its agent sweep had given up (bit 2 of the error word); no
@@ -953,7 +955,6 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
     }
 #endif
 #undef PM_CREATE
-    cudaFree(perm_d);
     h->iterations = 0;
     h->rho_pending = 0.5f;
     *out = h;

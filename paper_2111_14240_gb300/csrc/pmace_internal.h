@@ -191,8 +191,13 @@ cudaError_t launch_prep_amps(const void* amps_in, int amp_f16, const float* scal
                              int nblocks, cudaStream_t s);
 cudaError_t launch_reduce_partials(const double* partials, int nrows, int ncols, double* out,
                                    cudaStream_t s);
-cudaError_t launch_init_stack(float2* q, const float2* init, float2 cval, const int2* offs,
+// init == NULL: the constant sqrt(*sumsq / jd) (0 where jd is 0).
+cudaError_t launch_init_stack(float2* q, const float2* init, const double* sumsq, double jd, const int2* offs,
                               int J, int np, int n2, cudaStream_t s);
+// 1/d ((0, 0) where |d| <= absent or d = 0) and |d|^kappa of P probe values,
+// in double, rounded once.
+cudaError_t launch_probe_tables(const float2* d, float2* dinv, float* wk, int P, double kappa, double absent,
+                                cudaStream_t s);
 cudaError_t launch_patches_from_state(const float2* q, const float2* xbar, const int2* offs,
                                       float2* v, int J, int np, int n1, int n2, float two_rho,
                                       int* err, cudaStream_t s);

@@ -326,10 +326,12 @@ cudaError_t launch_reduce_partials(const double* partials, int nrows, int ncols,
 // ---------------------------------------------------------------------------
 // Algorithm 1 initialisation w = v = [P_j x^(0)]_j, stored as the pending
 // stack q (the consensus image starts at 0, so v = q + 2 rho P xbar = q).
-// init == NULL means the constant image cval.
+// init == NULL means the energy-matched constant sqrt(*sumsq / jd).
 // ---------------------------------------------------------------------------
-__global__ void init_stack_kernel(float2* __restrict__ q, const float2* __restrict__ init, float2 cval,
+__global__ void init_stack_kernel(float2* __restrict__ q, const float2* __restrict__ init,
+                                  const double* __restrict__ sumsq, double jd,
                                   const int2* __restrict__ offs, int J, int np, int n2) {
+    const float2 cval = make_float2(init == nullptr && jd > 0.0 ? (float)sqrt(*sumsq / jd) : 0.f, 0.f);
     const size_t P = (size_t)np * np;
     const size_t total = (size_t)J * P;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -345,9 +347,27 @@ __global__ void init_stack_kernel(float2* __restrict__ q, const float2* __restri
     }
 }
 
-cudaError_t launch_init_stack(float2* q, const float2* init, float2 cval, const int2* offs, int J,
+cudaError_t launch_init_stack(float2* q, const float2* init, const double* sumsq, double jd, const int2* offs, int J,
                               int np, int n2, cudaStream_t s) {
-    init_stack_kernel<<<1216, 256, 0, s>>>(q, init, cval, offs, J, np, n2);
+    init_stack_kernel<<<1216, 256, 0, s>>>(q, init, sumsq, jd, offs, J, np, n2);
+    return cudaGetLastError();
+}
+
+// Probe tables.  On the device because the 16384 powers of a 128 x 128 probe
+// took the host 0.3 ms of a job's creation.
+__global__ void __launch_bounds__(128)
+probe_tables_kernel(const float2* __restrict__ d, float2* __restrict__ dinv, float* __restrict__ wk, int P, double kappa,
+                    double absent) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= P) return;
+    const double re = d[i].x, im = d[i].y, m2 = re * re + im * im, m = sqrt(m2);
+    wk[i] = (float)pow(m, kappa);
+    dinv[i] = m > absent && m > 0.0 ? make_float2((float)(re / m2), (float)(-im / m2)) : make_float2(0.f, 0.f);
+}
+
+cudaError_t launch_probe_tables(const float2* d, float2* dinv, float* wk, int P, double kappa, double absent,
+                                cudaStream_t s) {
+    probe_tables_kernel<<<(P + 127) / 128, 128, 0, s>>>(d, dinv, wk, P, kappa, absent);
     return cudaGetLastError();
 }
 
