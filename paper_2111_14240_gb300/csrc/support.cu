@@ -31,14 +31,70 @@ namespace pmace {
 // that brings the counter to the tile's unit count resets it to 0, reads
 // the slots back from L2 in ascending order and writes the pixels.
 // ---------------------------------------------------------------------------
-template <int MODE, int TH>
+// A window of the chunk in shared memory: its stack values and its corner.
+struct __align__(16) StagedWindow {
+    const float2* src;
+    int row, col;
+};
+constexpr int kNoRow = -(1 << 29);   // corner of a window that covers no pixel
+
+// The n windows of a chunk (padded to a multiple of U with windows that cover
+// nothing) into the sums of pixels (py0 + r * RS, px), U windows at a time so
+// that U * RPT loads are in flight per thread; the accumulation still runs
+// over ascending window index.  NP is the window size at compile time: the
+// rows of a thread are then one address and constants, which with the
+// pointers staged took the instructions per window and pixel slot from 25 to
+// about half.
+template <int MODE, int NP, int U, int RPT, int RS, typename Acc>
+__device__ __forceinline__ void gather_chunk(const GatherArgs& g, const StagedWindow* win, int n, int px, int py0,
+                                             uint64_t pol, Acc (&acc)[RPT]) {
+#pragma unroll 1
+    for (int k0 = 0; k0 < n; k0 += U) {
+        float wgt[U][RPT];
+        float2 val[U][RPT];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const StagedWindow s = win[k0 + k];
+            const int lx = px - s.col, ly = py0 - s.row, e = (int)((unsigned)ly * NP + (unsigned)lx);
+            const float* w = g.wk + e;
+            const float2* v = s.src + e;
+            const bool inx = (unsigned)lx < (unsigned)NP;
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                wgt[k][r] = 0.f;
+                val[k][r] = make_float2(0.f, 0.f);
+                if (inx && (unsigned)(ly + r * RS) < (unsigned)NP) {
+                    wgt[k][r] = __ldg(w + r * RS * NP);
+                    if constexpr (MODE == 1) val[k][r] = ld_nc_l2_hint(v + r * RS * NP, pol);
+                    else if constexpr (MODE == 2) val[k][r] = __ldg(v + r * RS * NP);
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                if (wgt[k][r] != 0.f) {
+                    if constexpr (MODE == 0) {
+                        acc[r] += (double)wgt[k][r];
+                    } else {
+                        acc[r].x = fmaf(wgt[k][r], val[k][r].x, acc[r].x);
+                        acc[r].y = fmaf(wgt[k][r], val[k][r].y, acc[r].y);
+                    }
+                }
+            }
+        }
+    }
+}
+
+template <int MODE, int TH, int U>
 __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit) {
     constexpr int TW = kGatherTileW;
     constexpr int NT = gather_threads(TH);
     constexpr int RPT = kGatherRowsPerThread;       // rows per thread
     static_assert(NT >= kGatherStage, "one thread stages one window of a chunk");
-    __shared__ int s_i[kGatherStage];
-    __shared__ int2 s_o[kGatherStage];
+    static_assert(NT >= U, "one thread pads one window");
+    __shared__ StagedWindow s_win[kGatherStage + U];
     __shared__ int s_last;
 
     const int4 un = __ldg(g.units + unit);          // (tile, lb, le, slot)
@@ -78,59 +134,22 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
             int2 o = __ldg(g.offs + i);
             if (bad_i || o.x < 0 || o.x > g.n1 - np || o.y < 0 || o.y > g.n2 - np) {
                 atomicOr(g.err, kErrBoundsBit);
-                o = make_int2(-(1 << 29), -(1 << 29));
+                o = make_int2(kNoRow, kNoRow);
             }
-            s_i[threadIdx.x] = i;
-            s_o[threadIdx.x] = o;
 #else
-            s_i[threadIdx.x] = i;
-            s_o[threadIdx.x] = __ldg(g.offs + i);
+            const int2 o = __ldg(g.offs + i);
 #endif
+            s_win[threadIdx.x] = StagedWindow{g.src + (size_t)i * P, o.x, o.y};
         }
+        if (threadIdx.x < U) s_win[n + threadIdx.x] = StagedWindow{nullptr, kNoRow, kNoRow};
         __syncthreads();
-        // Windows are taken U at a time so that U * RPT loads are in flight
-        // per thread; the accumulation still runs over ascending window index.
-        // (U = 3 keeps 8 CTAs an SM; U = 4 with 7 was 4 % slower on the
-        // 8192 x 8192 / 64009-window consensus, U = 8 with 4 CTAs 30 %.)
-        constexpr int U = 3;
-        for (int k0 = 0; k0 < n; k0 += U) {
-            float wgt[U][RPT];
-            float2 val[U][RPT];
-#pragma unroll
-            for (int k = 0; k < U; ++k) {
-                const bool have = k0 + k < n;
-                const int i = have ? s_i[k0 + k] : 0;
-                const int2 o = have ? s_o[k0 + k] : make_int2(-(1 << 29), -(1 << 29));
-                const int lx = px - o.y;
-                const bool inx = have && (unsigned)lx < (unsigned)np;
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) {
-                    const int py = ty0 + grp + r * (NT / TW);
-                    const int ly = py - o.x;
-                    wgt[k][r] = 0.f;
-                    val[k][r] = make_float2(0.f, 0.f);
-                    if (inx && (unsigned)ly < (unsigned)np) {
-                        const int e = ly * np + lx;
-                        wgt[k][r] = __ldg(g.wk + e);
-                        if constexpr (MODE == 1) val[k][r] = ld_nc_l2_hint(g.src + (size_t)i * P + e, pol_first);
-                        else if constexpr (MODE == 2) val[k][r] = __ldg(g.src + (size_t)i * P + e);
-                    }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < U; ++k) {
-#pragma unroll
-                for (int r = 0; r < RPT; ++r) {
-                    if (wgt[k][r] != 0.f) {
-                        if constexpr (MODE == 0) {
-                            acc[r] += (double)wgt[k][r];
-                        } else {
-                            acc[r].x = fmaf(wgt[k][r], val[k][r].x, acc[r].x);
-                            acc[r].y = fmaf(wgt[k][r], val[k][r].y, acc[r].y);
-                        }
-                    }
-                }
-            }
+        const int py0 = ty0 + grp;
+        constexpr int RS = NT / TW;
+        switch (np) {
+            case 32: gather_chunk<MODE, 32, U, RPT, RS>(g, s_win, n, px, py0, pol_first, acc); break;
+            case 64: gather_chunk<MODE, 64, U, RPT, RS>(g, s_win, n, px, py0, pol_first, acc); break;
+            case 128: gather_chunk<MODE, 128, U, RPT, RS>(g, s_win, n, px, py0, pol_first, acc); break;
+            default: gather_chunk<MODE, 256, U, RPT, RS>(g, s_win, n, px, py0, pol_first, acc); break;
         }
     }
     if (un.w >= 0) {                                 // tile split over several units
@@ -195,29 +214,42 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
     }
 }
 
-template <int MODE, int TH>
+template <int MODE, int TH, int U>
 __global__ void __launch_bounds__(gather_threads(TH)) gather_kernel(const __grid_constant__ GatherArgs g) {
-    gather_body<MODE, TH>(g, blockIdx.x);
+    gather_body<MODE, TH, U>(g, blockIdx.x);
 }
 
 // Several jobs' units in one launch: CTA k gathers unit work[k].y of job work[k].x.
-template <int MODE, int TH>
+template <int MODE, int TH, int U>
 __global__ void __launch_bounds__(gather_threads(TH))
 gather_kernel_batched(const GatherArgs* __restrict__ descs, const int2* __restrict__ work) {
     const int2 w = work[blockIdx.x];
-    gather_body<MODE, TH>(descs[w.x], w.y);
+    gather_body<MODE, TH, U>(descs[w.x], w.y);
 }
 
-template <int MODE>
-static cudaError_t launch_gather(const GatherArgs& g, int nunits, int tile_h, cudaStream_t s) {
-    if (nunits <= 0) return cudaSuccess;
+// Windows taken at a time: kGatherWide where the launch leaves the GPU mostly
+// empty, so that the round trips of a unit's windows set its duration (63
+// units of 16 windows: 12.0 us against 15.4), else kGatherU, whose registers
+// let 8 CTAs share an SM (four at a time, with 7 CTAs, was 4 % slower on the
+// 64009-window consensus, eight, with 4 CTAs, 30 %).
+constexpr int kGatherU = 3, kGatherWide = 8;
+constexpr int kGatherWideUnits = 304;   // two CTAs an SM
+
+template <int MODE, int U>
+static cudaError_t launch_gather_u(const GatherArgs& g, int nunits, int tile_h, cudaStream_t s) {
     switch (tile_h) {
-        case 8: gather_kernel<MODE, 8><<<nunits, gather_threads(8), 0, s>>>(g); break;
-        case 16: gather_kernel<MODE, 16><<<nunits, gather_threads(16), 0, s>>>(g); break;
-        case 32: gather_kernel<MODE, 32><<<nunits, gather_threads(32), 0, s>>>(g); break;
+        case 8: gather_kernel<MODE, 8, U><<<nunits, gather_threads(8), 0, s>>>(g); break;
+        case 16: gather_kernel<MODE, 16, U><<<nunits, gather_threads(16), 0, s>>>(g); break;
+        case 32: gather_kernel<MODE, 32, U><<<nunits, gather_threads(32), 0, s>>>(g); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+template <int MODE>
+static cudaError_t launch_gather(const GatherArgs& g, int nunits, int tile_h, cudaStream_t s) {
+    if (nunits <= 0) return cudaSuccess;
+    if (MODE != 0 && nunits <= kGatherWideUnits) return launch_gather_u<MODE, kGatherWide>(g, nunits, tile_h, s);
+    return launch_gather_u<MODE, kGatherU>(g, nunits, tile_h, s);
 }
 cudaError_t launch_gather_weights(const GatherArgs& g, int n, int th, cudaStream_t s) { return launch_gather<0>(g, n, th, s); }
 cudaError_t launch_gather_consensus(const GatherArgs& g, int n, int th, cudaStream_t s) { return launch_gather<1>(g, n, th, s); }
@@ -227,9 +259,9 @@ cudaError_t launch_gather_consensus_batched(const GatherArgs* descs, const int2*
                                             cudaStream_t s) {
     if (nunits <= 0) return cudaSuccess;
     switch (tile_h) {
-        case 8: gather_kernel_batched<1, 8><<<nunits, gather_threads(8), 0, s>>>(descs, work); break;
-        case 16: gather_kernel_batched<1, 16><<<nunits, gather_threads(16), 0, s>>>(descs, work); break;
-        case 32: gather_kernel_batched<1, 32><<<nunits, gather_threads(32), 0, s>>>(descs, work); break;
+        case 8: gather_kernel_batched<1, 8, kGatherU><<<nunits, gather_threads(8), 0, s>>>(descs, work); break;
+        case 16: gather_kernel_batched<1, 16, kGatherU><<<nunits, gather_threads(16), 0, s>>>(descs, work); break;
+        case 32: gather_kernel_batched<1, 32, kGatherU><<<nunits, gather_threads(32), 0, s>>>(descs, work); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
