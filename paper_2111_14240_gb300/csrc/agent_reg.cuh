@@ -62,6 +62,7 @@
 #pragma once
 
 #include "agent_xpose.cuh"
+#include "pdl.cuh"
 
 namespace pmace {
 
@@ -258,10 +259,8 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
             bulk_load(region_s + (uint32_t)(N * sizeof(float2)) * (uint32_t)l, a.q + ((size_t)j * N + w + W * l) * N,
                       (uint32_t)(N * sizeof(float2)), bar);
     };
-    load_stack(j0);
-
     // v in columns 0..63 of the warp's lanes, 1/d in 64..127.  The tables are
-    // loaded all at once, while the first window's stack is on its way.
+    // loaded all at once, while the kernel before this one ends.
     const uint32_t tm_v = *s_tm + ((uint32_t)(32 * (w & 3)) << 16) + 128u * (uint32_t)(w >> 2), tm_i = tm_v + 64u;
     const float2* __restrict__ d_l2 = a.probe + w * N + l;   // value e = CC rr + cc at W N rr + 32 cc
     bool absent = false;   // whether one of the thread's pixels has its probe value treated as absent (1/d = 0)
@@ -285,6 +284,8 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
 #pragma unroll
     for (int e = 0; e < G::kDSmem; ++e) s_d[e * T + t] = x[e];
     tmem_wait_st();
+    pdl_wait();   // the stacks and the consensus image from here on
+    load_stack(j0);
 
     constexpr float inv_n = 1.0f / (float)N;
     const bool first = a.first != 0;
@@ -605,7 +606,6 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
             bulk_load(region_s, a.q + (size_t)j * (N * N), kCopyBytes, bar);
         }
     };
-    if (j0 < a.J) load_stack(j0);
     if (t == 0) {
         const float two_rho = 2.0f * a.rho_cur, inv1pa = 1.0f / (1.0f + a.alpha), two_rho_prev = 2.0f * a.rho_prev;
         const float keep = 1.0f - inv1pa, data = inv1pa * (1.0f / (float)N);   // as in reg_body
@@ -638,6 +638,8 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
     const bool wu = a.u != nullptr;
     const size_t n2 = (size_t)a.n2;
     auto xbar_at = [&](int2 off) { return a.xbar + (size_t)off.x * a.n2 + off.y + l; };
+    pdl_wait();   // the stacks and the consensus image from here on
+    if (j0 < a.J) load_stack(j0);
     float2 x[32];
     {
         const float2* __restrict__ xr = xbar_at(off_next);
@@ -859,8 +861,7 @@ cudaError_t agent_reg(const AgentArgs* a, int amp_f16, cudaStream_t s, AgentPlan
     if (a == nullptr) return reg_query(e, G::T, G::kSmem, G::kPer, info);
     if (e != cudaSuccess) return e;
     if (a->wpc <= 0) return cudaErrorInvalidValue;
-    fn<<<(unsigned)((a->J + a->wpc - 1) / a->wpc), G::T, G::kSmem, s>>>(*a);
-    return cudaGetLastError();
+    return pdl_launch(a->overlap != 0, fn, (unsigned)((a->J + a->wpc - 1) / a->wpc), G::T, G::kSmem, s, *a);
 }
 
 template <int N>
@@ -881,8 +882,7 @@ inline cudaError_t agent_reg32(const AgentArgs* a, int amp_f16, cudaStream_t s, 
     if (a == nullptr) return reg_query(e, G::T, G::kSmem, G::kPer, info);
     if (e != cudaSuccess) return e;
     if (a->wpc <= 0) return cudaErrorInvalidValue;
-    fn<<<(unsigned)((a->J + a->wpc - 1) / a->wpc), G::T, G::kSmem, s>>>(*a);
-    return cudaGetLastError();
+    return pdl_launch(a->overlap != 0, fn, (unsigned)((a->J + a->wpc - 1) / a->wpc), G::T, G::kSmem, s, *a);
 }
 
 inline cudaError_t agent_reg32_batched(const AgentArgs* descs, const int2* work, int nctas, int amp_f16,

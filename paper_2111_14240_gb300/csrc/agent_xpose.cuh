@@ -48,6 +48,7 @@
 
 #include "agent.cuh"
 #include "cache_hints.cuh"
+#include "pdl.cuh"
 #include "tmem.cuh"
 
 #include <type_traits>
@@ -362,6 +363,7 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
             prefetch_l2(static_cast<const char*>(a.y) + ((size_t)jw * N * N + (size_t)rank * 16 * T) * (AMP ? 2 : 4),
                         16 * T * (AMP ? 2 : 4));
     };
+    pdl_wait();   // the stacks and the consensus image from here on
     prefetch_window(j0);
 
     // the window corner is loaded a window ahead, so the consensus loads of
@@ -706,6 +708,7 @@ cudaLaunchConfig_t xpose_config(K, int nclusters, cudaStream_t s, cudaLaunchAttr
     attr[0].val.clusterDim.x = G::C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();   // counted in by a launch that overlaps (AgentArgs::overlap)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cfg;
@@ -736,7 +739,7 @@ cudaError_t agent_xpose(const AgentArgs* a, int amp_f16, cudaStream_t s, AgentPl
         info->smem_bytes = G::kSmemLaunch;
         info->max_clusters = 0;
         if (e == cudaSuccess && et == cudaSuccess) {
-            cudaLaunchAttribute attr[1];
+            cudaLaunchAttribute attr[2];
             cudaLaunchConfig_t cfg = xpose_config<N>(twin, 64, nullptr, attr);
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, twin, &cfg) == cudaSuccess) info->max_clusters = n;
@@ -748,8 +751,9 @@ cudaError_t agent_xpose(const AgentArgs* a, int amp_f16, cudaStream_t s, AgentPl
     if (e != cudaSuccess) return e;
     if (a->wpc <= 0) return cudaErrorInvalidValue;
     const int nclusters = (a->J + a->wpc - 1) / a->wpc;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = xpose_config<N>(fn, nclusters, s, attr);
+    if (a->overlap) cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, fn, *a);
 }
 
@@ -762,7 +766,7 @@ cudaError_t agent_xpose_batched(const AgentArgs* descs, const int2* work, int nc
         amp_f16 ? agent_xpose_kernel_batched<N, 1> : agent_xpose_kernel_batched<N, 0>;
     cudaError_t e = xpose_attributes(fn, G::kSmemLaunch, G::C);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = xpose_config<N>(fn, nclusters, s, attr);
     return cudaLaunchKernelEx(&cfg, fn, descs, work);
 }

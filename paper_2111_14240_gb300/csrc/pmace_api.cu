@@ -621,6 +621,7 @@ pmace_status launch_iteration(pmace_job* h, float alpha, float rho, cudaStream_t
     AgentArgs a = agent_args(h, alpha, rho);
     a.residual = residual ? 1 : 0;
     a.spectrum = spectrum;
+    a.overlap = small_consensus(h->nunits) ? 1 : 0;
     const bool from_q = consensus_from_q(rho);
     const GatherArgs g = consensus_args(h, rho);
     if (events) PM_CUDA(h, record_pair(h->ev_agent, h->n_agent, true, s));

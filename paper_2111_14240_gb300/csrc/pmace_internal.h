@@ -50,6 +50,7 @@ struct AgentArgs {
     int residual;           // 1: write the residual partial sums (else they are left untouched)
     int keep;               // 1: store the stack the gather reads next (q, or u where it is written) with the
                             // L2 evict-last hint (the stack fits about twice the L2)
+    int overlap;            // 1: the launch may start while the kernel before it ends (pdl.cuh)
     int wpc;                // windows per cluster (transposing-exchange variant)
     int* err;               // bit 2: a bounded device-side wait gave up; bit 3: a bounds check of the
                             // PMACE_DEBUG build failed
@@ -96,6 +97,9 @@ constexpr int kGatherRowsPerThread = 4;
 // slot = -1: the tile has one unit, which writes the result.
 // Windows of a unit are staged in shared memory kGatherStage at a time.
 constexpr int kGatherStage = 64;
+// Consensus launches of at most two CTAs an SM leave the GPU mostly empty:
+// they take more windows at a time and overlap with the kernels around them.
+constexpr bool small_consensus(int nunits) { return nunits <= 304; }
 __host__ __device__ constexpr int gather_threads(int tile_h) {
     return tile_h / kGatherRowsPerThread * kGatherTileW;
 }

@@ -84,7 +84,7 @@ struct Result {
 int64_t footprint(const pmace_dims& d, pmace_amp_format fmt) {
     const int64_t P = (int64_t)d.np * d.np, JP = (int64_t)d.J * P, NI = (int64_t)d.n1 * d.n2;
     // gather scratch: one slot of at most 32 x 32 pixels per unit of a split
-    // tile; the block length keeps the units near 3072 (a little over, where
+    // tile; the block length keeps the units near 2400 (a little over, where
     // the 8- and 32-row tiles cut differently than the 16-row ones)
     const int64_t per_window = (int64_t)(d.np / 8 + 2) * (d.np / 32 + 2);
     const int64_t slots = std::min<int64_t>(8192, (int64_t)d.J * per_window / 8);

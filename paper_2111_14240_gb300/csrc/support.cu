@@ -4,6 +4,7 @@
 // residual partials, and the stack initialisation of Algorithm 1.
 #include "pmace_internal.h"
 #include "cache_hints.cuh"
+#include "pdl.cuh"
 
 #include <cuda_fp16.h>
 
@@ -142,6 +143,7 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
             s_win[threadIdx.x] = StagedWindow{g.src + (size_t)i * P, o.x, o.y};
         }
         if (threadIdx.x < U) s_win[n + threadIdx.x] = StagedWindow{nullptr, kNoRow, kNoRow};
+        if (cb == un.y) pdl_wait();                 // the stack from here on
         __syncthreads();
         const int py0 = ty0 + grp;
         constexpr int RS = NT / TW;
@@ -152,6 +154,7 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
             default: gather_chunk<MODE, 256, U, RPT, RS>(g, s_win, n, px, py0, pol_first, acc); break;
         }
     }
+    if (un.y >= un.z) pdl_wait();                    // no window: the images are still read and written
     if (un.w >= 0) {                                 // tile split over several units
         Acc* mine = reinterpret_cast<Acc*>(g.scratch) + (size_t)un.w * (TH * TW);
 #pragma unroll
@@ -233,22 +236,28 @@ gather_kernel_batched(const GatherArgs* __restrict__ descs, const int2* __restri
 // let 8 CTAs share an SM (four at a time, with 7 CTAs, was 4 % slower on the
 // 64009-window consensus, eight, with 4 CTAs, 30 %).
 constexpr int kGatherU = 3, kGatherWide = 8;
-constexpr int kGatherWideUnits = 304;   // two CTAs an SM
+
+// The consensus of a small iteration starts while its agent sweep ends (pdl.cuh).
+template <int MODE, typename K>
+static cudaError_t gather_launch(K fn, int nunits, int threads, cudaStream_t s, const GatherArgs& g) {
+    if constexpr (MODE == 1) return pdl_launch(small_consensus(nunits), fn, (unsigned)nunits, (unsigned)threads, 0, s, g);
+    fn<<<nunits, threads, 0, s>>>(g);
+    return cudaGetLastError();
+}
 
 template <int MODE, int U>
 static cudaError_t launch_gather_u(const GatherArgs& g, int nunits, int tile_h, cudaStream_t s) {
     switch (tile_h) {
-        case 8: gather_kernel<MODE, 8, U><<<nunits, gather_threads(8), 0, s>>>(g); break;
-        case 16: gather_kernel<MODE, 16, U><<<nunits, gather_threads(16), 0, s>>>(g); break;
-        case 32: gather_kernel<MODE, 32, U><<<nunits, gather_threads(32), 0, s>>>(g); break;
+        case 8: return gather_launch<MODE>(gather_kernel<MODE, 8, U>, nunits, gather_threads(8), s, g);
+        case 16: return gather_launch<MODE>(gather_kernel<MODE, 16, U>, nunits, gather_threads(16), s, g);
+        case 32: return gather_launch<MODE>(gather_kernel<MODE, 32, U>, nunits, gather_threads(32), s, g);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 template <int MODE>
 static cudaError_t launch_gather(const GatherArgs& g, int nunits, int tile_h, cudaStream_t s) {
     if (nunits <= 0) return cudaSuccess;
-    if (MODE != 0 && nunits <= kGatherWideUnits) return launch_gather_u<MODE, kGatherWide>(g, nunits, tile_h, s);
+    if (MODE != 0 && small_consensus(nunits)) return launch_gather_u<MODE, kGatherWide>(g, nunits, tile_h, s);
     return launch_gather_u<MODE, kGatherU>(g, nunits, tile_h, s);
 }
 cudaError_t launch_gather_weights(const GatherArgs& g, int n, int th, cudaStream_t s) { return launch_gather<0>(g, n, th, s); }
