@@ -68,8 +68,8 @@ WORKLOADS = {
 }
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "agent_traffic.json")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2111_14240_gb300", "csrc", f)
-                  for f in ("agent.cuh", "agent_xpose.cuh", "agent_pair.cuh", "cache_hints.cuh", "tmem.cuh",
-                            "fft_smem.cuh", "pmace_internal.h")]
+                  for f in ("agent.cuh", "agent_reg.cuh", "agent_xpose.cuh", "agent_pair.cuh", "cache_hints.cuh",
+                            "tmem.cuh", "pdl.cuh", "fft_smem.cuh", "pmace_internal.h")]
 
 
 def kernel_hash() -> str:
@@ -90,15 +90,17 @@ def kernel_hash() -> str:
 
 def agent_bytes_per_patch(np_: int, amp_bytes: int = 4) -> int:
     """Algorithmic HBM bytes of the agent sweep per window: read q, read y,
-    write u, write q (complex64 = 8 B, amplitude 4 or 2 B per pixel).  The
-    window of the consensus image it reads is L2-resident and not counted."""
-    return np_ * np_ * (8 + amp_bytes + 8 + 8)
+    write q (complex64 = 8 B, amplitude 4 or 2 B per pixel; the consensus is
+    taken from q at the benchmark's rho).  The window of the consensus image
+    it reads is L2-resident and not counted."""
+    return np_ * np_ * (8 + amp_bytes + 8)
 
 
 def iteration_bytes(np_: int, J: int, n1: int, n2: int, amp_bytes: int = 4) -> int:
     """Algorithmic bytes of one whole iteration: the agent sweep plus the
-    gather's read of u and its image traffic (write xbar, read Lambda^-1)."""
-    return J * (agent_bytes_per_patch(np_, amp_bytes) + np_ * np_ * 8) + n1 * n2 * (8 + 4)
+    gather's read of q and its image traffic (read and write x_hat, write xbar,
+    read Lambda^-1)."""
+    return J * (agent_bytes_per_patch(np_, amp_bytes) + np_ * np_ * 8) + n1 * n2 * (8 + 8 + 8 + 4)
 
 
 # ------------------------------------------------------------------ clocks

@@ -48,17 +48,17 @@
 // agent_xpose.cuh: a warp whose wait for its copies gives up sets bit 2 of
 // *err, and the CTA's threads agree at the next block barrier and stop.
 //
-// Measured (GB300, FP16 amplitudes, one sweep): 64009 windows 5.38 ms against
-// 7.10 for the cluster form (3.5 TB/s of the 18 bytes a pixel the sweep must
-// move: read q and y, write q), 14641 windows 1.22 against 1.66 ms, 900 windows
-// (FP32) 91 against 125 us; 3600 windows of 64 x 64 92 against 160 us (against
+// Measured (GB300, FP16 amplitudes, one sweep): 64009 windows 5.12 ms against
+// 7.10 for the cluster form (3.7 TB/s of the 18 bytes a pixel the sweep must
+// move: read q and y, write q), 14641 windows 1.17 against 1.66 ms, 900 windows
+// (FP32) 90 against 125 us; 3600 windows of 64 x 64 92 against 160 us (against
 // the cluster form), of 32 x 32 24 against 41 us (against one CTA a window in
 // place).  What bounds the 128 x 128 sweep: about 13.5 k of a window's 26 k
 // cycles are instruction issue (75 % of it on the FP32 pipes), 8 k the
 // shared-memory passes, and the store of 128 KB takes 4.1 k at the 32 bytes a
 // cycle an SM can store; the block barriers keep the warps in step, so these
 // overlap only in part.  Bulk stores of q' with plain loads of q, the other
-// way round from what is built, were no faster (1.24 ms).
+// way round from what is built, were no faster (1.24 ms against 1.22 then).
 #pragma once
 
 #include "agent_xpose.cuh"
