@@ -158,9 +158,12 @@ pmace_status pmace_kernel_times(pmace_handle h, double* agent_ms, int64_t* agent
  * staged in shared memory, how many clusters the device holds at once, how
  * the 2-D DFT is split over the cluster (exchange 0: an in-place cross-CTA
  * butterfly stage; 1: a transposing exchange of 16 x 16 blocks between the
- * Np / 16 CTAs, which then run their column transforms locally; 2: the same
+ * Np / 16 CTAs, which then run their column transforms locally, or, where
+ * cluster is 1, exchanges between the warps of the one CTA that holds the
+ * window in registers; 2: the same
  * exchange with two windows per cluster at a time in packed FP32 lanes) and
- * the windows each cluster processes; for the consensus gather the image
+ * the windows each cluster processes (for 32 x 32 probes in registers: each
+ * CTA, a window a warp at a time); for the consensus gather the image
  * tile shape. */
 typedef struct {
     int32_t cluster, threads, smem_bytes, tile_h, tile_w;

@@ -689,7 +689,7 @@ pmace_status switch_plan(pmace_job* h, int variant, int tile_h, cudaStream_t s) 
         return fail(h, PMACE_ERR_INVALID_ARG, "tile_h %d not in {8, 16, 32}", tile_h);
     if (variant != h->variant) {
         AgentPlanInfo info{};
-        const int impl = agent_impl(np, variant, J);
+        const int impl = agent_impl(np, variant, J, h->amp_f16);
         if (agent_entry(np, nullptr, impl, h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
             cudaGetLastError();
             return fail(h, PMACE_ERR_UNSUPPORTED_SIZE, "agent variant %d cannot run on this device", variant);
@@ -812,7 +812,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         for (int i = 0; i < kAgentVariants && chosen < 0; ++i) {
             const int v = (v0 + i) % kAgentVariants;
             AgentPlanInfo info{};
-            if (agent_entry(np, nullptr, agent_impl(np, v, J), h->amp_f16, s, &info) == cudaSuccess && info.launchable) {
+            if (agent_entry(np, nullptr, agent_impl(np, v, J, h->amp_f16), h->amp_f16, s, &info) == cudaSuccess && info.launchable) {
                 h->plan = info;
                 chosen = v;
             }
@@ -821,7 +821,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         if (chosen < 0)
             return bail(fail(h, PMACE_ERR_UNSUPPORTED_SIZE, "no launchable agent plan for np=%d", np));
         h->variant = chosen;
-        h->impl = agent_impl(np, chosen, J);
+        h->impl = agent_impl(np, chosen, J, h->amp_f16);
         h->cluster = agent_variant_of(np, h->impl).cluster;
         h->wpc = windows_per_cluster(np, h->impl, J, h->plan);
     }
@@ -1060,7 +1060,7 @@ pmace_status pmace_autotune(pmace_handle h, const pmace_step* step, int32_t iter
     // agent variants at the current tile height, then tile heights for the best variant
     for (int v = 0; v < kAgentVariants && st == PMACE_OK; ++v) {
         AgentPlanInfo info{};
-        if (agent_entry(h->dims.np, nullptr, agent_impl(h->dims.np, v, h->dims.J), h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
+        if (agent_entry(h->dims.np, nullptr, agent_impl(h->dims.np, v, h->dims.J, h->amp_f16), h->amp_f16, s, &info) != cudaSuccess || !info.launchable) {
             cudaGetLastError();
             continue;
         }

@@ -149,11 +149,18 @@ __host__ __device__ constexpr int default_agent_variant(int np) { return np >= 6
 // 29.7, 342 46 / 64, 900 91 / 125; 64 x 64: J = 100 14.1 / 12.7, 168 15.2 / 14.6,
 // 374 19.3 / 24.9, 750 30 / 39, 3600 92 / 159.  The 32 x 32 register sweep (a
 // window a warp) takes the place of the in-place sweep with one CTA a window.
+// 64 x 64 and 128 x 128 windows with FP32 amplitudes keep the cluster sweep.
+// It finishes the row axis before it starts the columns, which confines the
+// rounding of the last seven levels to strong columns; the register sweep
+// ends the row axis last, and its rounding reaches the weak coefficients: over
+// 100 iterations of the converging 900-window workload at peak 1e6 the error
+// over the well-illuminated pixels is 1.2 % from the 64-bit run's, against
+// 0.6 %. Under FP16 amplitudes their own 2^-11 steps are far above either.
 constexpr int kReg128MinWindows = 72;
 constexpr int kReg64MinWindows = 180;
-__host__ __device__ constexpr int agent_impl(int np, int v, int J) {
+__host__ __device__ constexpr int agent_impl(int np, int v, int J, int amp_f16) {
     if (np == 32) return v == 1 ? kRegImpl : v;
-    return v == 4 && ((np == 128 && J >= kReg128MinWindows) || (np == 64 && J >= kReg64MinWindows)) ? kRegImpl : v;
+    return v == 4 && amp_f16 && ((np == 128 && J >= kReg128MinWindows) || (np == 64 && J >= kReg64MinWindows)) ? kRegImpl : v;
 }
 
 // Geometry of one agent plan (probe size, CTAs per patch).
