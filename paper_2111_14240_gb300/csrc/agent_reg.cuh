@@ -103,6 +103,15 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                  : "memory");
 }
 
+// Bounded wait of a whole warp: the lanes poll one by one and may reach the
+// limit at different polls, so they vote, and all of them take the way of a
+// wait that gave up if any did.  What follows a wait is warp-wide (.sync.aligned
+// tensor-memory accesses, full-mask shuffles and warp barriers); the vote also
+// brings the lanes back together for it.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* err) {
+    return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, err));
+}
+
 // A read-only load that stays where it is written (the compiler moves plain
 // ones up, which costs the registers they are meant to wait for).
 __device__ __forceinline__ float2 ld_here(const float2* p) {
@@ -333,7 +342,7 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
         const size_t wbase = (size_t)j * N * N;
         // ---- S0 + S1: the consensus values are in x (loaded by the update
         // of the previous window as it freed the registers)
-        const bool got = mbar_wait_bounded(bar, parity, a.err);
+        const bool got = mbar_wait_warp(bar, parity, a.err);
         {
             const float2* st = reinterpret_cast<const float2*>(region) + l;
             const float2 trp2 = make_float2(s_const[1].x, s_const[1].y);
@@ -399,7 +408,7 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
         if (__syncthreads_or(!got)) {
             // a wait that gave up stops the CTA; its warp's copies may still
             // be in flight: one more (bounded) wait before shared memory goes
-            if (!got) mbar_wait_bounded(bar, parity, a.err);
+            if (!got) mbar_wait_warp(bar, parity, a.err);
             break;
         }
         parity ^= 1u;
@@ -663,8 +672,8 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
         }
         const size_t wbase = (size_t)j * N * N;
         // ---- S0 + S1, and the first radix-32 pass (rows)
-        if (!mbar_wait_bounded(bar, parity, a.err)) {
-            mbar_wait_bounded(bar, parity, a.err);   // the warp stops: see reg_body
+        if (!mbar_wait_warp(bar, parity, a.err)) {
+            mbar_wait_warp(bar, parity, a.err);   // the warp stops: see reg_body
             break;
         }
         parity ^= 1u;
