@@ -112,12 +112,25 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
     return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, err));
 }
 
-// A read-only load that stays where it is written (the compiler moves plain
-// ones up, which costs the registers they are meant to wait for).
+// A load of a probe table (read-only while the kernel runs) that stays where it
+// is written (the compiler moves plain ones up, which costs the registers they
+// are meant to wait for).
 __device__ __forceinline__ float2 ld_here(const float2* p) {
     float2 v;
     asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
+}
+
+// The consensus values of a thread's next window.  A launch that may start while
+// the gather before it still writes the image (LIVE, pdl.cuh) takes plain loads.
+// Where the kernel before has ended, read-only ones: with plain loads, which stay
+// in order with the stores around them, the 64009-window sweep of 128 x 128
+// windows spills 150 bytes more a thread (two iterations 15.9 ms against 14.9,
+// 3600 windows of 64 x 64 276 us against 272).
+template <bool LIVE>
+__device__ __forceinline__ float2 ld_next(const float2* p) {
+    if constexpr (LIVE) return ld_live(p);
+    else return ld_here(p);
 }
 
 // Pass 1 forward on x[CC rr + cc]: radix CC over cc with the lane's twiddles
@@ -218,8 +231,9 @@ __device__ __forceinline__ void named_arrive(int id, int count) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// Windows j0, j0 + step, ... below J of the job `a` on one CTA.
-template <int N, int AMP>
+// Windows j0, j0 + step, ... below J of the job `a` on one CTA.  LIVE: the
+// launch may start while the kernel before it runs.
+template <int N, int AMP, bool LIVE>
 __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const int step) {
     using G = RegGeom<N>;
     constexpr int T = G::T, W = G::W, CC = G::CC, RR = G::RR, IR = G::IR, KB = G::KB;
@@ -327,9 +341,9 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
     // where the thread's consensus values of the window at `off` start
     auto xbar_at = [&](int2 off) { return a.xbar + (size_t)(off.x + w) * a.n2 + off.y + l; };
     {
-        const float2* __restrict__ xr = xbar_at(off_next);
+        const float2* xr = xbar_at(off_next);
 #pragma unroll
-        for (int e = 0; e < 32; ++e) x[e] = __ldg(xr + (e / CC) * rows_w + 32 * (e % CC));
+        for (int e = 0; e < 32; ++e) x[e] = ld_live(xr + (e / CC) * rows_w + 32 * (e % CC));
     }
 #pragma unroll 1
     for (int j = j0; j < a.J; j += step) {
@@ -511,8 +525,8 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
             const uint64_t pol_q = wu ? l2_policy_evict_first() : pol_next;
             float2* qr = a.q + wbase + w * N + l;
             float2* __restrict__ ur = a.u + wbase + w * N + l;
-            const float2* __restrict__ xr = xbar_at(off);
-            const float2* __restrict__ xn = xbar_at(off_next);
+            const float2* xr = xbar_at(off);
+            const float2* xn = xbar_at(off_next);
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
                 uint32_t rv[8], ri[8];
@@ -533,7 +547,7 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int e = 4 * g + k;
-                        residual_sums(first ? v[k] : __ldg(xr + (e / CC) * rows_w + 32 * (e % CC)), wv[k], acc_z, acc_w);
+                        residual_sums(first ? v[k] : ld_live(xr + (e / CC) * rows_w + 32 * (e % CC)), wv[k], acc_z, acc_w);
                     }
                 }
 #pragma unroll
@@ -544,7 +558,7 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    x[4 * g + k] = ld_here(xn + 32 * ((4 * g + k) % CC));
+                    x[4 * g + k] = ld_next<LIVE>(xn + 32 * ((4 * g + k) % CC));
                     if ((4 * g + k) % CC == CC - 1) xn += rows_w;
                 }
             }
@@ -651,9 +665,9 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
     if (j0 < a.J) load_stack(j0);
     float2 x[32];
     {
-        const float2* __restrict__ xr = xbar_at(off_next);
+        const float2* xr = xbar_at(off_next);
 #pragma unroll
-        for (int e = 0; e < 32; ++e) x[e] = __ldg(xr + e * n2);
+        for (int e = 0; e < 32; ++e) x[e] = ld_live(xr + e * n2);
     }
     tmem_fence_before_sync();
     absent = __syncthreads_or(absent);
@@ -758,8 +772,8 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
             const uint64_t pol_q = wu ? l2_policy_evict_first() : pol_next;
             float2* qr = a.q + wbase + l;
             float2* __restrict__ ur = a.u + wbase + l;
-            const float2* __restrict__ xr = xbar_at(off);
-            const float2* __restrict__ xn = xbar_at(off_next);
+            const float2* xr = xbar_at(off);
+            const float2* xn = xbar_at(off_next);
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
                 uint32_t rv[8];
@@ -780,7 +794,7 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
                 if (res) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        residual_sums(first ? v[k] : __ldg(xr + (4 * g + k) * n2), wv[k], acc_z, acc_w);
+                        residual_sums(first ? v[k] : ld_live(xr + (4 * g + k) * n2), wv[k], acc_z, acc_w);
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -790,7 +804,7 @@ __device__ __forceinline__ void reg32_body(const AgentArgs& a, const int cta, co
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    x[4 * g + k] = ld_here(xn);
+                    x[4 * g + k] = ld_live(xn);
                     xn += n2;
                 }
             }
@@ -833,9 +847,9 @@ agent_reg32_kernel_batched(const AgentArgs* __restrict__ descs, const int2* __re
 // CTAs are always within a few windows of one another in scan order and the
 // consensus image they read stays in L2 (with contiguous runs the 64009-window
 // sweep of 128 x 128 windows took 7.24 ms instead of 5.62).
-template <int N, int AMP>
+template <int N, int AMP, bool LIVE>
 __global__ void __launch_bounds__(RegGeom<N>::T, RegGeom<N>::kPer) agent_reg_kernel(const __grid_constant__ AgentArgs a) {
-    reg_body<N, AMP>(a, (int)blockIdx.x, (int)gridDim.x);
+    reg_body<N, AMP, LIVE>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // Several jobs: CTA k takes the share of job work[k].x that starts at window
@@ -845,7 +859,7 @@ __global__ void __launch_bounds__(RegGeom<N>::T, RegGeom<N>::kPer)
 agent_reg_kernel_batched(const AgentArgs* __restrict__ descs, const int2* __restrict__ work) {
     const int2 wk = work[blockIdx.x];
     const AgentArgs& a = descs[wk.x];
-    reg_body<N, AMP>(a, wk.y / a.wpc, (a.J + a.wpc - 1) / a.wpc);
+    reg_body<N, AMP, false>(a, wk.y / a.wpc, (a.J + a.wpc - 1) / a.wpc);
 }
 
 // Query (a == nullptr: fills info; a "cluster" is one CTA) or launch
@@ -865,12 +879,14 @@ inline cudaError_t reg_query(cudaError_t e, int threads, int smem, int per, Agen
 template <int N>
 cudaError_t agent_reg(const AgentArgs* a, int amp_f16, cudaStream_t s, AgentPlanInfo* info) {
     using G = RegGeom<N>;
-    void (*fn)(const AgentArgs) = amp_f16 ? agent_reg_kernel<N, 1> : agent_reg_kernel<N, 0>;
+    const bool live = a != nullptr && a->overlap != 0;
+    void (*fn)(const AgentArgs) = live ? (amp_f16 ? agent_reg_kernel<N, 1, true> : agent_reg_kernel<N, 0, true>)
+                                       : (amp_f16 ? agent_reg_kernel<N, 1, false> : agent_reg_kernel<N, 0, false>);
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem);
     if (a == nullptr) return reg_query(e, G::T, G::kSmem, G::kPer, info);
     if (e != cudaSuccess) return e;
     if (a->wpc <= 0) return cudaErrorInvalidValue;
-    return pdl_launch(a->overlap != 0, fn, (unsigned)((a->J + a->wpc - 1) / a->wpc), G::T, G::kSmem, s, *a);
+    return pdl_launch(live, fn, (unsigned)((a->J + a->wpc - 1) / a->wpc), G::T, G::kSmem, s, *a);
 }
 
 template <int N>

@@ -387,14 +387,14 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
             const int row = row0 + k;
             const float2* qr = a.q + wbase + (size_t)row * N;
             const float2* __restrict__ dr = a.probe + (size_t)row * N;
-            const float2* __restrict__ xr = a.xbar + (size_t)(off.x + row) * a.n2 + off.y;
+            const float2* xr = a.xbar + (size_t)(off.x + row) * a.n2 + off.y;
             // all stack loads first (one memory round trip), then the
             // L2-resident consensus and probe values
             float2 x[r1];
 #pragma unroll
             for (int t = 0; t < r1; ++t) x[t] = qr[b + S1 * t];
 #pragma unroll
-            for (int t = 0; t < r1; ++t) x[t] = mann_close2(x[t], __ldg(xr + b + S1 * t), trp2);
+            for (int t = 0; t < r1; ++t) x[t] = mann_close2(x[t], ld_live(xr + b + S1 * t), trp2);
             if constexpr (kTm) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {   // keep v for the copy-out
@@ -599,7 +599,7 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
                 Dft<r1, true>::run(x);
                 float2* qr = a.q + wbase + (size_t)row * N;   // read (S0) and overwritten (S5) by this thread only
                 float2* __restrict__ ur = a.u + wbase + (size_t)row * N;
-                const float2* __restrict__ xr = a.xbar + (size_t)(off.x + row) * a.n2 + off.y;
+                const float2* xr = a.xbar + (size_t)(off.x + row) * a.n2 + off.y;
                 // in quarters: the loads of a quarter are issued together
                 constexpr int H = r1 / 4;
                 if constexpr (kTm) tmem_wait_st();   // v of the copy-in has landed
@@ -615,7 +615,7 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
                         for (int t = 0; t < H; ++t) {
                             qv[t] = make_float2(__uint_as_float(rv[2 * t]), __uint_as_float(rv[2 * t + 1]));
                             dv[t] = make_float2(__uint_as_float(rd[2 * t]), __uint_as_float(rd[2 * t + 1]));
-                            if constexpr (kRes) xv[t] = __ldg(xr + b + S1 * (h0 + t));
+                            if constexpr (kRes) xv[t] = ld_live(xr + b + S1 * (h0 + t));
                         }
                     } else {
                         const float2* __restrict__ dr = a.dinv + (size_t)row * N;
@@ -623,7 +623,7 @@ __device__ __forceinline__ void xpose_body(const AgentArgs& a, const int j0, con
                         for (int t = 0; t < H; ++t) {
                             const int s = b + S1 * (h0 + t);
                             qv[t] = qr[s];
-                            xv[t] = __ldg(xr + s);
+                            xv[t] = ld_live(xr + s);
                             dv[t] = __ldg(dr + s);
                         }
                     }

@@ -32,9 +32,9 @@ __device__ __forceinline__ void st_l2_hint(float2* ptr, float2 v, uint64_t pol) 
     asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(ptr), "f"(v.x), "f"(v.y), "l"(pol)
                  : "memory");
 }
-__device__ __forceinline__ float2 ld_nc_l2_hint(const float2* ptr, uint64_t pol) {
+__device__ __forceinline__ float2 ld_l2_hint(const float2* ptr, uint64_t pol) {
     float2 v;
-    asm volatile("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(ptr), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(ptr), "l"(pol));
     return v;
 }
 __device__ __forceinline__ float ld_nc_l2_hint(const float* ptr, uint64_t pol) {

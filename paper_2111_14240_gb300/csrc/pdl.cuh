@@ -25,6 +25,16 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A load of what an earlier kernel of the stream wrote (the consensus image),
+// for kernels that may be launched with the attribute: they are resident while
+// that kernel still writes, which read-only loads (__ldg, ld.global.nc) do not
+// allow, and the compiler may move those over pdl_wait.
+__device__ __forceinline__ float2 ld_live(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 inline cudaLaunchAttribute pdl_attribute() {
     cudaLaunchAttribute a = {};
     a.id = cudaLaunchAttributeProgrammaticStreamSerialization;

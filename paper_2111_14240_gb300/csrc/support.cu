@@ -66,7 +66,7 @@ __device__ __forceinline__ void gather_chunk(const GatherArgs& g, const StagedWi
                 val[k][r] = make_float2(0.f, 0.f);
                 if (inx && (unsigned)(ly + r * RS) < (unsigned)NP) {
                     wgt[k][r] = __ldg(w + r * RS * NP);
-                    if constexpr (MODE == 1) val[k][r] = ld_nc_l2_hint(v + r * RS * NP, pol);
+                    if constexpr (MODE == 1) val[k][r] = ld_l2_hint(v + r * RS * NP, pol);
                     else if constexpr (MODE == 2) val[k][r] = __ldg(v + r * RS * NP);
                 }
             }

@@ -34,3 +34,37 @@ def test_register_sweep_lanes_agree_on_a_bounded_wait():
     for body in ("reg_body", "reg32_body"):
         assert function(src, body).count("mbar_wait_warp(") == 2
     assert "mbar_try_wait" not in src
+
+
+# kernels that a launch may start while the kernel before them still writes, and
+# the names by which they read what that kernel writes
+OVERLAPPED = [("agent_reg.cuh", "reg_body", r"x[rn]"), ("agent_reg.cuh", "reg32_body", r"x[rn]"),
+              ("agent_xpose.cuh", "xpose_body", r"xr"), ("support.cu", "gather_chunk", r"v")]
+
+
+def test_overlapped_kernels_read_live_data_by_plain_loads():
+    """Read-only loads (__ldg, ld.global.nc, const restrict pointers) are for
+    data that no one writes while the kernel is resident: under dependent
+    launch the consensus image and the stack are not."""
+    for name, body, var in OVERLAPPED:
+        src = function(source(name), body)
+        reads = re.findall(r"(\w+)\(%s(?: \+[^;]*?)?[,)]" % var, src)
+        if name == "support.cu":   # the readout (mode 2) is launched without overlap
+            src = re.sub(r"else if constexpr \(MODE == 2\)[^;]*;", "", src)
+            reads = re.findall(r"(\w+)\(v \+ ", src)
+        reads = [r for r in reads if r != "ld_live" and r != "ld_l2_hint"]
+        assert not reads, (body, reads)
+        assert not re.search(r"__restrict__\s+%s\b" % var, src), body
+    for name, fn in (("pdl.cuh", "ld_live"), ("cache_hints.cuh", "ld_l2_hint")):
+        asm = function(source(name), fn)
+        assert "asm volatile" in asm and ".nc" not in asm
+    # the loads of the next window are read-only ones only in the kernel that is
+    # launched without overlap
+    reg = source("agent_reg.cuh")
+    assert re.search(r"if constexpr \(LIVE\) return ld_live\(p\)", function(reg, "ld_next"))
+    assert re.search(r"live \? \(amp_f16 \? agent_reg_kernel<N, 1, true>[^;]*: \(amp_f16 \? agent_reg_kernel<N, 1, false>[^;]*;",
+                     reg) and "pdl_launch(live, fn," in reg and "reg_body<N, AMP, false>(a, wk.y" in reg
+    # pdl_wait comes before the first of these reads
+    for name, body, var in OVERLAPPED[:3]:
+        src = function(source(name), body)
+        assert src.index("pdl_wait()") < min(src.index(f"{f}(") for f in ("ld_live",) if f"{f}(" in src)
