@@ -53,6 +53,7 @@ struct pmace_job {
     int64_t iterations = 0;
     float rho_pending = 0.5f;
     bool xhat_valid = false;  // xhat holds x_hat of the current (q, xbar)
+    bool replayable = false;  // a caller's graph may change the state: xhat_valid says nothing
 
     std::vector<int32_t> offs_host;   // window corners, for rebuilding the overlap lists
 

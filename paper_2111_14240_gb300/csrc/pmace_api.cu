@@ -583,6 +583,14 @@ static bool user_capture(const pmace_job* h, cudaStream_t s) {
     return cap == cudaStreamCaptureStatusActive && s != h->capture_stream;
 }
 
+// Every call that changes the state comes by here first.  What it records under
+// a caller's capture changes q and xbar whenever the graph is replayed, of which
+// the host learns nothing: from then on the kept readout image is not trusted
+// and every readout gathers.
+static void note_capture(pmace_job* h, cudaStream_t s) {
+    if (user_capture(h, s)) h->replayable = true;
+}
+
 // x_hat of the current state into dst.
 static cudaError_t readout(const pmace_job* h, float2* dst, cudaStream_t s) {
     GatherArgs g = gather_args(h);
@@ -594,18 +602,17 @@ static cudaError_t readout(const pmace_job* h, float2* dst, cudaStream_t s) {
 }
 
 cudaError_t ensure_xhat(pmace_job* h, cudaStream_t s) {
-    // Under a caller's stream capture the readout is always recorded: the
-    // state may have been replaced by the time the graph is replayed.
-    const bool captured = user_capture(h, s);
-    if (h->xhat_valid && !captured) return cudaSuccess;
+    if (h->xhat_valid && !h->replayable) return cudaSuccess;
     const cudaError_t e = readout(h, h->xhat, s);
-    if (e == cudaSuccess && !captured) h->xhat_valid = true;
+    if (e == cudaSuccess && !user_capture(h, s)) h->xhat_valid = true;   // a recorded readout has not run
     return e;
 }
 
 // x_hat of the current state into device memory of the caller's.
 static cudaError_t readout_to(const pmace_job* h, float2* dst, cudaStream_t s) {
-    if (!h->xhat_valid || user_capture(h, s)) return readout(h, dst, s);
+    // recorded in a caller's graph, the readout is always the gather: the state
+    // may have been replaced by the time the graph is replayed
+    if (!h->xhat_valid || h->replayable || user_capture(h, s)) return readout(h, dst, s);
     return launch_copy_image(dst, h->xhat, (int64_t)h->dims.n1 * h->dims.n2, s);
 }
 }  // namespace pmace
@@ -973,6 +980,7 @@ pmace_status pmace_iterate(pmace_handle h, int32_t n, const pmace_step* step, vo
     if (!(rho > 0.f && rho < 1.f)) return fail(h, PMACE_ERR_INVALID_ARG, "rho must be in (0, 1) (got %g)", rho);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (n == 0) return PMACE_OK;
+    note_capture(h, s);
     if (consensus_from_q(rho)) PM_CUDA(h, ensure_xhat(h, s));
     int32_t done = 0;
     // Iterations that open with the pending rho of an earlier call (or the
@@ -1128,6 +1136,7 @@ pmace_status pmace_debug_spectra(pmace_handle h, const pmace_step* step, float* 
                     h->variant);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float2* dst = reinterpret_cast<float2*>(out);
+    note_capture(h, s);
     if (consensus_from_q(step->rho)) PM_CUDA(h, ensure_xhat(h, s));
     pmace_status st = launch_iteration(h, step->alpha, step->rho, s, false, true, dst);
     if (st != PMACE_OK) return st;
@@ -1213,6 +1222,7 @@ pmace_status pmace_set_state(pmace_handle h, const float* q, const float* xbar,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const size_t JP = (size_t)h->dims.J * h->dims.np * h->dims.np, NI = (size_t)h->dims.n1 * h->dims.n2;
+    note_capture(h, s);
     PM_CUDA(h, cudaMemcpyAsync(h->q, q, JP * sizeof(float2), k, s));
     PM_CUDA(h, cudaMemcpyAsync(h->xbar, xbar, NI * sizeof(float2), k, s));
     if (!on_device) PM_CUDA(h, cudaStreamSynchronize(s));
