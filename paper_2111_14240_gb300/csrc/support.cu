@@ -197,9 +197,12 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
         } else {
             const float li = __ldg(g.laminv + p);
             float2 v = make_float2(acc[r].x * li, acc[r].y * li);
+            // a pixel without weight (li = 0, acc = 0) is 0 in both images,
+            // whatever a state set by the caller holds there
+            auto weighted = [li](float2 a) { return make_float2(li != 0.f ? a.x : 0.f, li != 0.f ? a.y : 0.f); };
             if constexpr (MODE == 1) {
                 if (g.xhat) {
-                    const float2 xh = g.xhat[p];
+                    const float2 xh = weighted(g.xhat[p]);
                     const float k = g.c2 * li;
                     const float2 xb =
                         make_float2(fmaf(-k, acc[r].x, g.c1 * xh.x), fmaf(-k, acc[r].y, g.c1 * xh.y));
@@ -208,7 +211,7 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
                 }
             }
             if constexpr (MODE == 2) {
-                const float2 xb = __ldg(g.xbar_in + p);
+                const float2 xb = weighted(__ldg(g.xbar_in + p));
                 v.x = fmaf(g.two_rho, xb.x, v.x);
                 v.y = fmaf(g.two_rho, xb.y, v.y);
             }
