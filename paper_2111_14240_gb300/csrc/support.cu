@@ -203,9 +203,11 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
             if constexpr (MODE == 1) {
                 if (g.xhat) {
                     const float2 xh = weighted(g.xhat[p]);
-                    const float k = g.c2 * li;
-                    const float2 xb =
-                        make_float2(fmaf(-k, acc[r].x, g.c1 * xh.x), fmaf(-k, acc[r].y, g.c1 * xh.y));
+                    // Lambda^-1 (c2 acc), not (c2 Lambda^-1) acc: in the far tail of
+                    // a probe (Lambda below 2^-127) Lambda^-1 is finite and c2
+                    // times it is not
+                    const float2 s = make_float2(g.c2 * acc[r].x, g.c2 * acc[r].y);
+                    const float2 xb = make_float2(fmaf(-li, s.x, g.c1 * xh.x), fmaf(-li, s.y, g.c1 * xh.y));
                     g.xhat[p] = make_float2(fmaf(g.two_rho, xb.x, v.x), fmaf(g.two_rho, xb.y, v.y));
                     v = xb;
                 }

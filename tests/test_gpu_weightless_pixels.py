@@ -1,5 +1,6 @@
-"""Pixels the probe does not weight: outside the scan the images read 0 whatever
-a state that was set holds there."""
+"""Pixels the probe does not weight, or hardly: outside the scan the images read
+0 whatever a state that was set holds there, and where Lambda is near the
+smallest single-precision numbers an iteration stays finite."""
 import numpy as np
 import pytest
 
@@ -41,3 +42,22 @@ def test_uncovered_pixels_of_a_set_state_read_zero(np_, J, rho):
         out.append(images)
     for images in out[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(images, out[0]))
+
+
+@pytest.mark.parametrize("rho", [0.3, 0.5, 0.7])
+def test_probe_tail_at_the_smallest_weights(rho):
+    """|d|^2 = 4e-39 in two columns of the probe, alone there: Lambda^-1 is
+    finite and (1/rho) Lambda^-1 is not.  The data say nothing about those
+    pixels (1/d makes 1e11 of a rounding error), but they stay finite and the
+    others are what the oracle gives."""
+    from tests.gpu_helpers import TOL_ITER, random_start, rel_l2, run_gpu, run_oracle
+    w = _workload(32, 1)
+    w.probe[:, :2] = 6.3e-20
+    x0 = random_start(w)
+    g = run_gpu(w, 2, 0.5, rho, kappa=2.0, init=x0)
+    o = run_oracle(w, 2, 0.5, rho, kappa=2.0, x0=x0)
+    assert np.isfinite(g["x_hat"]).all() and np.isfinite(g["v"]).all()
+    lit = np.abs(w.probe) > 0.1 * np.abs(w.probe).max()
+    assert rel_l2(g["v"][:, lit], o["v"][:, lit]) < 2 * TOL_ITER
+    (r, c), n = w.offsets[0], 32
+    assert rel_l2(g["x_hat"][r:r + n, c:c + n][lit], o["x_hat"][r:r + n, c:c + n][lit]) < 2 * TOL_ITER
