@@ -231,13 +231,13 @@ __device__ __forceinline__ void named_arrive(int id, int count) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// Windows j0, j0 + step, ... below J of the job `a` on one CTA.  LIVE: the
-// launch may start while the kernel before it runs.
-template <int N, int AMP, bool LIVE>
+// Windows j0, j0 + step, ... below J of the job `a` on one CTA, with
+// FP16 amplitudes (agent_impl).  LIVE: the launch may start while the kernel
+// before it runs.
+template <int N, bool LIVE>
 __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const int step) {
     using G = RegGeom<N>;
     constexpr int T = G::T, W = G::W, CC = G::CC, RR = G::RR, IR = G::IR, KB = G::KB;
-    constexpr int NCH = AMP ? 1 : 2;          // 16-byte chunks of eight amplitudes
     constexpr uint32_t kCopyBytes = RR * N * sizeof(float2);
 
     extern __shared__ float4 smem_raw[];
@@ -320,8 +320,8 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
     auto prefetch = [&](int j) {
         if (l < RR) prefetch_l2(a.q + ((size_t)j * N + w + W * l) * N, (uint32_t)(N * sizeof(float2)));
         else if (l == RR) {
-            constexpr uint32_t yb = 1024 * (AMP ? 2 : 4);
-            prefetch_l2(static_cast<const char*>(a.y) + (size_t)j * N * N * (AMP ? 2 : 4) + (size_t)w * yb, yb);
+            constexpr uint32_t yb = 1024 * sizeof(__half);
+            prefetch_l2(static_cast<const char*>(a.y) + (size_t)j * N * N * sizeof(__half) + (size_t)w * yb, yb);
         }
     };
     // Where a window takes sixteen warps, four groups of four take turns (a
@@ -410,14 +410,13 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
 #pragma unroll
             for (int p = 0; p < 16; ++p) mine[32 * p] = make_float4(x[2 * p].x, x[2 * p].y, x[2 * p + 1].x, x[2 * p + 1].y);
         }
-        uint4 raw[4 * NCH];
-        float yscale = 1.0f;
+        uint4 raw[4];   // eight codes each
+        const float yscale = __ldg(a.yscale + j);
         {
-            const uint4* yp = reinterpret_cast<const uint4*>(static_cast<const char*>(a.y) + wbase * (AMP ? 2 : 4)) + t;
+            const uint4* yp = reinterpret_cast<const uint4*>(static_cast<const char*>(a.y) + wbase * sizeof(__half)) + t;
             const uint64_t pol_first = l2_policy_evict_first();
 #pragma unroll
-            for (int k = 0; k < 4 * NCH; ++k) raw[k] = ld_nc_l2_hint(yp + k * T, pol_first);
-            if constexpr (AMP == 1) yscale = __ldg(a.yscale + j);
+            for (int k = 0; k < 4; ++k) raw[k] = ld_nc_l2_hint(yp + k * T, pol_first);
         }
         if (__syncthreads_or(!got)) {
             // a wait that gave up stops the CTA; its warp's copies may still
@@ -460,9 +459,9 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
 #pragma unroll
                     for (int h = 0; h < IR * B / 8; ++h) {   // eight at a time: registers
                         float yv[8];
-                        unpack_amps8<AMP>(raw + NCH * (IR * k0 / 8 + h), yv);
+                        unpack_amps8<1>(raw + IR * k0 / 8 + h, yv);
                         replace_magnitudes<kRes>(reinterpret_cast<float2(&)[8]>(z[IR * k0 + 8 * h]), yv, inv_n, acc_d, acc_y,
-                                                 AMP == 1 ? yscale : 1.0f);
+                                                 yscale);
                     }
 #pragma unroll
                     for (int b = 0; b < B; ++b) Dft<IR, true>::run(reinterpret_cast<float2(&)[IR]>(z[IR * (k0 + b)]));
@@ -519,7 +518,7 @@ __device__ __forceinline__ void reg_body(const AgentArgs& a, const int j0, const
         {
             const float4 c0 = s_const[0], c1 = s_const[1];
             const float2 keep2 = make_float2(c0.x, c0.y), m2rho2 = make_float2(c0.z, c0.w);
-            const float ds = AMP == 1 ? c1.z * yscale : c1.z;
+            const float ds = c1.z * yscale;
             const float2 data2 = make_float2(ds, ds);
             const uint64_t pol_next = a.keep ? l2_policy_evict_last() : l2_policy_evict_normal();
             const uint64_t pol_q = wu ? l2_policy_evict_first() : pol_next;
@@ -847,19 +846,19 @@ agent_reg32_kernel_batched(const AgentArgs* __restrict__ descs, const int2* __re
 // CTAs are always within a few windows of one another in scan order and the
 // consensus image they read stays in L2 (with contiguous runs the 64009-window
 // sweep of 128 x 128 windows took 7.24 ms instead of 5.62).
-template <int N, int AMP, bool LIVE>
+template <int N, bool LIVE>
 __global__ void __launch_bounds__(RegGeom<N>::T, RegGeom<N>::kPer) agent_reg_kernel(const __grid_constant__ AgentArgs a) {
-    reg_body<N, AMP, LIVE>(a, (int)blockIdx.x, (int)gridDim.x);
+    reg_body<N, LIVE>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // Several jobs: CTA k takes the share of job work[k].x that starts at window
 // work[k].y / wpc, every ceil(J / wpc)-th window.
-template <int N, int AMP>
+template <int N>
 __global__ void __launch_bounds__(RegGeom<N>::T, RegGeom<N>::kPer)
 agent_reg_kernel_batched(const AgentArgs* __restrict__ descs, const int2* __restrict__ work) {
     const int2 wk = work[blockIdx.x];
     const AgentArgs& a = descs[wk.x];
-    reg_body<N, AMP, false>(a, wk.y / a.wpc, (a.J + a.wpc - 1) / a.wpc);
+    reg_body<N, false>(a, wk.y / a.wpc, (a.J + a.wpc - 1) / a.wpc);
 }
 
 // Query (a == nullptr: fills info; a "cluster" is one CTA) or launch
@@ -880,8 +879,8 @@ template <int N>
 cudaError_t agent_reg(const AgentArgs* a, int amp_f16, cudaStream_t s, AgentPlanInfo* info) {
     using G = RegGeom<N>;
     const bool live = a != nullptr && a->overlap != 0;
-    void (*fn)(const AgentArgs) = live ? (amp_f16 ? agent_reg_kernel<N, 1, true> : agent_reg_kernel<N, 0, true>)
-                                       : (amp_f16 ? agent_reg_kernel<N, 1, false> : agent_reg_kernel<N, 0, false>);
+    if (!amp_f16) return cudaErrorInvalidValue;   // agent_impl
+    void (*fn)(const AgentArgs) = live ? agent_reg_kernel<N, true> : agent_reg_kernel<N, false>;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem);
     if (a == nullptr) return reg_query(e, G::T, G::kSmem, G::kPer, info);
     if (e != cudaSuccess) return e;
@@ -893,7 +892,8 @@ template <int N>
 cudaError_t agent_reg_batched(const AgentArgs* descs, const int2* work, int nctas, int amp_f16, cudaStream_t s) {
     using G = RegGeom<N>;
     if (nctas <= 0) return cudaSuccess;
-    void (*fn)(const AgentArgs*, const int2*) = amp_f16 ? agent_reg_kernel_batched<N, 1> : agent_reg_kernel_batched<N, 0>;
+    if (!amp_f16) return cudaErrorInvalidValue;   // agent_impl
+    void (*fn)(const AgentArgs*, const int2*) = agent_reg_kernel_batched<N>;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, G::kSmem);
     if (e != cudaSuccess) return e;
     fn<<<(unsigned)nctas, G::T, G::kSmem, s>>>(descs, work);
