@@ -53,7 +53,8 @@ struct pmace_job {
     int64_t iterations = 0;
     float rho_pending = 0.5f;
     bool xhat_valid = false;  // xhat holds x_hat of the current (q, xbar)
-    bool replayable = false;  // a caller's graph may change the state: xhat_valid says nothing
+    bool replayable = false;  // a caller's graph may change the state: *xhat_ok takes the place of xhat_valid
+    int* xhat_ok = nullptr;   // kept on the device from then on; 0 before
 
     std::vector<int32_t> offs_host;   // window corners, for rebuilding the overlap lists
 

@@ -565,6 +565,7 @@ GatherArgs consensus_args(const pmace_job* h, float rho) {
     GatherArgs g = gather_args(h);
     g.out = h->xbar;
     g.src = h->u;
+    g.xhat_ok = h->replayable ? h->xhat_ok : nullptr;
     if (consensus_from_q(rho)) {
         g.src = h->q;
         g.keep = h->keep;
@@ -585,15 +586,26 @@ static bool user_capture(const pmace_job* h, cudaStream_t s) {
 
 // Every call that changes the state comes by here first.  What it records under
 // a caller's capture changes q and xbar whenever the graph is replayed, of which
-// the host learns nothing: from then on the kept readout image is not trusted
-// and every readout gathers.
+// the host learns nothing.  From then on the kernels note in *xhat_ok whether the
+// kept readout image is that of the state, and a call that needs it launches a
+// gather that does nothing if so: a replayed iteration pays a launch for it, not
+// a pass over the stack (900 windows of 128 x 128 174 us against 206).  A graph of
+// kGraphIters iterations captured earlier does not write the note; the iteration
+// that every call launches after it does.
 static void note_capture(pmace_job* h, cudaStream_t s) {
     if (user_capture(h, s)) h->replayable = true;
 }
 
-// x_hat of the current state into dst.
-static cudaError_t readout(const pmace_job* h, float2* dst, cudaStream_t s) {
+// A state from elsewhere, of which xhat is not the readout.
+static cudaError_t drop_xhat(pmace_job* h, cudaStream_t s) {
+    h->xhat_valid = false;
+    return h->replayable ? cudaMemsetAsync(h->xhat_ok, 0, sizeof(int), s) : cudaSuccess;
+}
+
+// x_hat of the current state into dst, where `skip` is given only if *skip is 0.
+static cudaError_t readout(const pmace_job* h, float2* dst, cudaStream_t s, const int* skip = nullptr) {
     GatherArgs g = gather_args(h);
+    g.skip = skip;
     g.src = h->q;
     g.xbar_in = h->xbar;
     g.out = dst;
@@ -602,7 +614,8 @@ static cudaError_t readout(const pmace_job* h, float2* dst, cudaStream_t s) {
 }
 
 cudaError_t ensure_xhat(pmace_job* h, cudaStream_t s) {
-    if (h->xhat_valid && !h->replayable) return cudaSuccess;
+    if (h->replayable) return readout(h, h->xhat, s, h->xhat_ok);
+    if (h->xhat_valid) return cudaSuccess;
     const cudaError_t e = readout(h, h->xhat, s);
     if (e == cudaSuccess && !user_capture(h, s)) h->xhat_valid = true;   // a recorded readout has not run
     return e;
@@ -876,7 +889,7 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
                      o_layout = lay.add<int>(P), o_tw = lay.add<float2>(np), o_offs = lay.add<int2>(J),
                      o_scale = lay.add<float>(h->amp_f16 ? J : 0),
                      o_part = lay.add<double>((size_t)J * kMaxCluster * 4 + kPrepBlocks), o_red = lay.add<double>(4),
-                     o_err = lay.add<int>(1);
+                     o_err = lay.add<int>(2);
         PM_CREATE(cudaMalloc(&h->mem, lay.bytes));
         h->bytes = (int64_t)lay.bytes;
         auto at = [&](size_t o, auto*& p) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(h->mem + o); };
@@ -896,11 +909,12 @@ pmace_status pmace_create(const pmace_dims* dims, const float* probe, const int3
         at(o_part, h->partials);
         at(o_red, h->red_out);
         at(o_err, h->err);
+        h->xhat_ok = h->err + 1;
     }
     pmace_status st = build_tables(h, probe_h, layout_d, s, keep);
     if (st == PMACE_OK) st = install_gather_tables(h, h->tile_h, s, &staged);
     if (st != PMACE_OK) return bail_sync(st);
-    PM_CREATE(cudaMemsetAsync(h->err, 0, sizeof(int), s));
+    PM_CREATE(cudaMemsetAsync(h->err, 0, 2 * sizeof(int), s));
 
     // amplitudes to kernel order (staged through u when they come from the host)
     const void* amps_dev = amps;
@@ -1036,9 +1050,9 @@ pmace_status pmace_autotune(pmace_handle h, const pmace_step* step, int32_t iter
     auto restore = [&]() -> cudaError_t {
         cudaError_t r = cudaMemcpyAsync(h->q, q0, JP * sizeof(float2), cudaMemcpyDeviceToDevice, s);
         if (r == cudaSuccess) r = cudaMemcpyAsync(h->xbar, x0, NI * sizeof(float2), cudaMemcpyDeviceToDevice, s);
+        if (r == cudaSuccess) r = drop_xhat(h, s);
         h->iterations = it0;
         h->rho_pending = rho0;
-        h->xhat_valid = false;
         return r;
     };
     // time `iters` iterations (after two untimed ones) of the current plan, ms per iteration
@@ -1225,10 +1239,10 @@ pmace_status pmace_set_state(pmace_handle h, const float* q, const float* xbar,
     note_capture(h, s);
     PM_CUDA(h, cudaMemcpyAsync(h->q, q, JP * sizeof(float2), k, s));
     PM_CUDA(h, cudaMemcpyAsync(h->xbar, xbar, NI * sizeof(float2), k, s));
+    PM_CUDA(h, drop_xhat(h, s));
     if (!on_device) PM_CUDA(h, cudaStreamSynchronize(s));
     h->iterations = info->iterations;
     h->rho_pending = info->rho_pending;
-    h->xhat_valid = false;
     return PMACE_OK;
 }
 

@@ -74,6 +74,8 @@ struct GatherArgs {
     float2* xhat;           // consensus from q: [n1][n2] readout image of the state before the iteration, replaced by
                             // that of the state after it; NULL: consensus from u
     float c1, c2;           // consensus from q: 1 / rho - 1 and 1 / rho
+    int* xhat_ok;           // consensus: set to whether the launch leaves xhat with the state (NULL: not kept)
+    const int* skip;        // readout: nothing is done where *skip is not 0 (NULL: always done)
     int keep;               // 1: src is read again soon and may stay in L2 (else it is read evict-first)
     float* lam_out;         // weight-image mode: Lambda^-1 written here
     int n1, n2, np, tiles_x;

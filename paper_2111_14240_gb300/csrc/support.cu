@@ -98,6 +98,9 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
     __shared__ StagedWindow s_win[kGatherStage + U];
     __shared__ int s_last;
 
+    if constexpr (MODE == 2) {
+        if (g.skip && __ldcg(g.skip)) return;       // the kept readout image is that of the state
+    }
     const int4 un = __ldg(g.units + unit);          // (tile, lb, le, slot)
 #ifdef PMACE_DEBUG
     // the unit must lie inside the tables (else the CTA flags it and stops)
@@ -155,6 +158,9 @@ __device__ __forceinline__ void gather_body(const GatherArgs& g, const int unit)
         }
     }
     if (un.y >= un.z) pdl_wait();                    // no window: the images are still read and written
+    if constexpr (MODE == 1) {
+        if (g.xhat_ok && unit == 0 && threadIdx.x == 0) *g.xhat_ok = g.xhat != nullptr;
+    }
     if (un.w >= 0) {                                 // tile split over several units
         Acc* mine = reinterpret_cast<Acc*>(g.scratch) + (size_t)un.w * (TH * TW);
 #pragma unroll

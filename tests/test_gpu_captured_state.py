@@ -83,3 +83,44 @@ def test_image_after_every_replay_of_set_state(np_, J):
         after.append(_host_image(rec))
     assert np.array_equal(after[0], after[1]) and not np.array_equal(after[0], want)
     rec.close()
+
+
+@pytest.mark.parametrize("np_,J", [(32, 40), (64, 30), (128, 20)])
+def test_replays_and_direct_calls_in_any_order(np_, J):
+    """Whether a call finds the readout image of the state or gathers it is
+    decided where the call runs: recorded and direct iterations on both sides of
+    rho = 1/2 and recorded and direct states in a random order, every one of
+    which begins and ends with rho = 1/2, against the direct calls alone."""
+    import torch
+
+    from paper_2111_14240_gb300 import pmace as pm
+    rec, ref = _job(np_, J), _job(np_, J)
+    state = []
+    for r in (rec, ref):
+        r.iterate(12, 0.5, 0.5)
+        q = torch.empty((J, np_, np_, 2), device="cuda")
+        xb = torch.empty((r.n1, r.n2, 2), device="cuda")
+        state.append((q, xb, pm.pmace_get_state(r.h, q, xb)))
+
+    def through_small_rho(r):
+        r.iterate(1, 0.5, 0.3)
+        r.iterate(1, 0.5, 0.5)
+
+    calls = [lambda r, k: r.iterate(1, 0.5, 0.5), lambda r, k: r.iterate(3, 0.5, 0.5),
+             lambda r, k: through_small_rho(r), lambda r, k: pm.pmace_set_state(r.h, *state[k])]
+    replays = [_captured(lambda c=c: c(rec, 0)) for c in calls]
+    calls.append(lambda r, k: r.iterate(11, 0.5, 0.5))   # replays a graph of the library's own: not recorded
+    rng = np.random.Generator(np.random.PCG64(np_))
+    for step in range(40):
+        i = int(rng.integers(len(calls)))
+        if i < len(replays) and rng.random() < 0.7:
+            replays[i]()
+        else:
+            calls[i](rec, 0)
+        calls[i](ref, 1)
+        if rng.random() < 0.5:
+            assert np.array_equal(_host_image(rec), ref.image().cpu().numpy()), step
+    assert np.array_equal(rec.image().cpu().numpy(), ref.image().cpu().numpy())
+    assert np.array_equal(rec.patches().cpu().numpy(), ref.patches().cpu().numpy())
+    rec.close()
+    ref.close()
