@@ -627,8 +627,8 @@ def run_ours(args):
         "config": {"workload": desc if not args.scan else f"{args.scan}x{args.scan} sub-raster of: {desc}",
                    "windows": J, "probe": np_, "image": [n1, n2],
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU",
-                   "l2": "no flush: per-step working set (q, u, y) is "
-                         f"{(J * np_ * np_ * (16 + amp_b)) / 1e9:.2f} GB > 129 MB L2",
+                   "l2": "no flush: per-step working set (q, y) is "
+                         f"{(J * np_ * np_ * (8 + amp_b)) / 1e9:.2f} GB > 129 MB L2",
                    "plan": plan},
         "roofline": roof,
         "kernels": {"agent_avg_ms": roof["avg_launch_ms"], "consensus_avg_ms": cons_avg_ms,

@@ -48,12 +48,11 @@
 // agent_xpose.cuh: a warp whose wait for its copies gives up sets bit 2 of
 // *err, and the CTA's threads agree at the next block barrier and stop.
 //
-// Measured (GB300, FP16 amplitudes, one sweep): 64009 windows 5.12 ms against
-// 7.10 for the cluster form (3.7 TB/s of the 18 bytes a pixel the sweep must
-// move: read q and y, write q), 14641 windows 1.17 against 1.66 ms, 900 windows
-// (FP32) 90 against 125 us; 3600 windows of 64 x 64 92 against 160 us (against
-// the cluster form), of 32 x 32 24 against 41 us (against one CTA a window in
-// place).  What bounds the 128 x 128 sweep: about 13.5 k of a window's 26 k
+// Measured (GB300, FP16 amplitudes, one sweep, against the cluster form): 64009
+// windows 5.07-5.21 against 7.19 ms (3.7 TB/s of the 18 bytes a pixel the sweep
+// must move: read q and y, write q), 14641 windows 1.17-1.20 against 1.68 ms, 900
+// windows 86 against 125 us; 3600 windows of 64 x 64 92 against 164 us, of 32 x 32
+// (both formats) 24 against 41 us for one CTA a window in place.  What bounds the 128 x 128 sweep: about 13.5 k of a window's 26 k
 // cycles are instruction issue (75 % of it on the FP32 pipes), 8 k the
 // shared-memory passes, and the store of 128 KB takes 4.1 k at the 32 bytes a
 // cycle an SM can store; the block barriers keep the warps in step, so these

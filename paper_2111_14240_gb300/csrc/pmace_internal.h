@@ -99,8 +99,9 @@ constexpr int kGatherRowsPerThread = 4;
 // slot = -1: the tile has one unit, which writes the result.
 // Windows of a unit are staged in shared memory kGatherStage at a time.
 constexpr int kGatherStage = 64;
-// Consensus launches of at most two CTAs an SM leave the GPU mostly empty:
-// they take more windows at a time and overlap with the kernels around them.
+// Consensus launches of at most two CTAs on each of the 152 SMs leave the GPU
+// mostly empty: they take more windows at a time and overlap with the kernels
+// around them.
 constexpr bool small_consensus(int nunits) { return nunits <= 304; }
 __host__ __device__ constexpr int gather_threads(int tile_h) {
     return tile_h / kGatherRowsPerThread * kGatherTileW;
@@ -146,10 +147,10 @@ __host__ __device__ constexpr int default_agent_variant(int np) { return np >= 6
 // The kernel that runs variant v for J windows of np x np.  The register
 // sweep takes a window a CTA (an SM for 128 x 128, a quarter of one for 64 x
 // 64), the cluster sweep spreads one over Np / 16 CTAs, which is the faster way
-// while the windows do not fill the SMs.  Agent sweep in us, register against
-// cluster, 128 x 128: J = 36 21 / 16.6, 64 21.3 / 20.7, 81 21.3 / 23.2, 120 22 /
-// 29.7, 342 46 / 64, 900 91 / 125; 64 x 64: J = 100 14.1 / 12.7, 168 15.2 / 14.6,
-// 374 19.3 / 24.9, 750 30 / 39, 3600 92 / 159.  The 32 x 32 register sweep (a
+// while the windows do not fill the SMs.  Agent sweep in us with FP16 amplitudes,
+// register against cluster, 128 x 128: J = 36 22.2 / 16.8, 64 22.3 / 20.8, 72 22.3 /
+// 22.2, 81 22.3 / 23.7, 120 21.9 / 29.9, 342 44 / 64, 900 86 / 125; 64 x 64: J = 100
+// 14.1 / 13.7, 168 15.8 / 14.8, 180 15.9 / 15.0, 374 20 / 26, 750 31 / 40, 3600 92 / 164.  The 32 x 32 register sweep (a
 // window a warp) takes the place of the in-place sweep with one CTA a window.
 // 64 x 64 and 128 x 128 windows with FP32 amplitudes keep the cluster sweep.
 // It finishes the row axis before it starts the columns, which confines the
@@ -157,7 +158,9 @@ __host__ __device__ constexpr int default_agent_variant(int np) { return np >= 6
 // ends the row axis last, and its rounding reaches the weak coefficients: over
 // 100 iterations of the converging 900-window workload at peak 1e6 the error
 // over the well-illuminated pixels is 1.2 % from the 64-bit run's, against
-// 0.6 %. Under FP16 amplitudes their own 2^-11 steps are far above either.
+// 0.6 %, and the bar is 1 %.  With FP16 amplitudes, against the 64-bit run on the
+// amplitudes the codes stand for, it stays within 0.35 % there (0.72 % for the
+// cluster sweep) and within 0.57 % (1.02 %) over the covered pixels.
 constexpr int kReg128MinWindows = 72;
 constexpr int kReg64MinWindows = 180;
 __host__ __device__ constexpr int agent_impl(int np, int v, int J, int amp_f16) {
